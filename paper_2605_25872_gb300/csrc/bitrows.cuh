@@ -32,6 +32,64 @@ __device__ __forceinline__ uint32_t rot_next(uint32_t v) {
     return (v >> 1) | ((v & 1u) << (L - 1));
 }
 
+// the W words of one colour row
+template <int W>
+__device__ __forceinline__ void load_words(const uint32_t *p, uint32_t (&w)[W]) {
+    if (W == 2) {
+        const uint2 v = *reinterpret_cast<const uint2 *>(p);
+        w[0] = v.x;
+        w[W - 1] = v.y;
+    } else {
+#pragma unroll
+        for (int j = 0; j < W; ++j) w[j] = p[j];
+    }
+}
+template <int W>
+__device__ __forceinline__ void store_words(uint32_t *p, const uint32_t (&w)[W]) {
+    if (W == 2) {
+        *reinterpret_cast<uint2 *>(p) = make_uint2(w[0], w[W - 1]);
+    } else {
+#pragma unroll
+        for (int j = 0; j < W; ++j) p[j] = w[j];
+    }
+}
+
+// Sign bits (1 = spin -1) of a natural x row whose colour-0 sites have x parity
+// p0: the two colour rows interleave (colour c holds x = 2m + p_c).
+// From the packed words of the byte layout: a multiply spreads a word's four
+// sign bits to every other bit (bits 25, 27, 29, 31 of the product).
+template <int L>
+__device__ __forceinline__ uint32_t row_of_words(const uint32_t (&w)[2][Geom<L>::W], int p0) {
+    constexpr int Lh = L / 2;
+    constexpr uint32_t H = 0x55555555u & ((1u << (2 * Lh - 1)) | ((1u << (2 * Lh - 1)) - 1u));
+    uint32_t row[2];
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+        uint32_t acc = 0;
+#pragma unroll
+        for (int j = 0; j < Geom<L>::W; ++j) acc |= (((w[c][j] & 0x80808080u) * 0x00041041u) >> 25) << (8 * j);
+        row[c] = acc & H;
+    }
+    return (row[0] << p0) | (row[1] << (p0 ^ 1));
+}
+// From the bit layout, row r.
+template <int L>
+__device__ __forceinline__ uint32_t row_of_bits(const uint32_t *S, int r, int p0) {
+    constexpr int W = Geom<L>::W;
+    uint32_t row[2];
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+        uint32_t n = 0;
+#pragma unroll
+        for (int j = 0; j < W; ++j) {
+            const int w = (c * Geom<L>::ROWS + r) * W + j;
+            n |= ((S[w >> 3] >> (4 * (w & 7))) & 0xFu) << (4 * j);
+        }
+        row[c] = spread_bits(n & ((1u << (L / 2)) - 1u));
+    }
+    return (row[0] << p0) | (row[1] << (p0 ^ 1));
+}
+
 // Row r = y + L z of the bit mask where lattices A and B differ (q_i = -1):
 // bit x set iff the spins at x + L r differ.  A and B in the storage layout
 // (BITS: the bit layout, else the byte layout).

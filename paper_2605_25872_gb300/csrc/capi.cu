@@ -264,19 +264,21 @@ pthr_status do_sweep(pthr_batch *b, int n_pt, int n_res, int first, int count, i
     return PTHR_OK;
 }
 
-// Threads per cluster-move block: about eight sites per thread, 128..512.
-int default_cluster_threads(int L) {
-    const int V = L * L * L;
-    int t = ((V / 8 + 31) / 32) * 32;
-    return t < 128 ? 128 : (t > 512 ? 512 : t);
-}
+constexpr int GPU_SMS = 152;   // GB300
 
+// Threads per cluster-move block: whole warps, each with one to eight pairs
+// (larger requests run as blocks of CLUSTER_MAX_THREADS).  By default the
+// largest block that still gives every SM two: a warp works alone until the
+// block's last barrier, so small launches spread better as small blocks.
 int cluster_threads_of(const pthr_batch *b) {
-    int threads = b->tuning.cluster_threads > 0 ? b->tuning.cluster_threads : default_cluster_threads(b->cfg.L);
-    const int V = b->cfg.L * b->cfg.L * b->cfg.L;
-    if (threads > ((V + 31) / 32) * 32) threads = ((V + 31) / 32) * 32;
-    if (threads < 32) threads = 32;
-    return (threads / 32) * 32;
+    int threads = CLUSTER_MAX_THREADS;
+    if (b->tuning.cluster_threads > 0) {
+        if (b->tuning.cluster_threads < threads) threads = b->tuning.cluster_threads;
+        return threads < 32 ? 32 : (threads / 32) * 32;
+    }
+    const int pairs = b->cfg.n_samples * b->dev.NPAIR * b->dev.n_acu;
+    while (threads > 32 && cluster_blocks_for(b->cfg.L, pairs, threads) < 2 * GPU_SMS) threads /= 2;
+    return threads;
 }
 
 pthr_status do_cluster(pthr_batch *b, int label_only, int32_t *labels) {
@@ -292,12 +294,8 @@ pthr_status do_cluster(pthr_batch *b, int label_only, int32_t *labels) {
     a.label_only = label_only;
     a.labels_out = labels;
     a.iter_cap = b->tuning.cluster_iter_cap;
-    int threads = b->tuning.cluster_threads > 0 ? b->tuning.cluster_threads : default_cluster_threads(b->cfg.L);
-    const int V = b->cfg.L * b->cfg.L * b->cfg.L;
-    if (threads > ((V + 31) / 32) * 32) threads = ((V + 31) / 32) * 32;
-    if (threads < 32) threads = 32;
-    threads = (threads / 32) * 32;
-    if (cluster_smem_bytes_for(b->cfg.L) > 200 * 1024)
+    const int threads = cluster_threads_of(b);
+    if (cluster_smem_bytes_for(b->cfg.L, threads) > 200 * 1024)
         return fail(b, PTHR_E_INVAL, "cluster block does not fit in shared memory");
     CUDA_TRY(b, launch_cluster(a, threads, b->stream), "cluster launch");
     return PTHR_OK;
@@ -527,7 +525,7 @@ PTHR_API pthr_status pthr_get_tuning(const pthr_batch *b, pthr_tuning *t) {
     t->pt_lattices_per_block = sh.K_pt;
     t->res_lattices_per_block = sh.K_res;
     t->sweep_threads = sh.threads;
-    t->cluster_threads = b->tuning.cluster_threads > 0 ? b->tuning.cluster_threads : default_cluster_threads(b->cfg.L);
+    t->cluster_threads = cluster_threads_of(b);
     t->cluster_iter_cap = b->tuning.cluster_iter_cap;
     return PTHR_OK;
 }
@@ -829,7 +827,10 @@ pthr_status group_fused_emcs(pthr_batch *const *batches, int n, cudaStream_t st,
     GroupSweepArgs gs{};
     GroupClusterArgs gc{};
     GroupBatchArgs gw{}, gm{};
-    int sw_threads = 32, cl_threads = 32, sw_blocks = 0, cl_blocks = 0, w_blocks = 0, m_blocks = 0, w_threads = 32;
+    int cl_threads = 32;   // one block size: the largest of the group
+    for (int i = 0; i < n; ++i)
+        if (cluster_threads_of(batches[i]) > cl_threads) cl_threads = cluster_threads_of(batches[i]);
+    int sw_threads = 32, sw_blocks = 0, cl_blocks = 0, w_blocks = 0, m_blocks = 0, w_threads = 32;
     size_t sw_smem = 0, cl_smem = 0, w_smem = 0, m_smem = 0;
     for (int ii = 0; ii < n; ++ii) {
         pthr_batch *b = batches[order[ii]];
@@ -853,10 +854,8 @@ pthr_status group_fused_emcs(pthr_batch *const *batches, int n, cudaStream_t st,
             gc.a[gc.n] = a;
             gc.off[gc.n] = cl_blocks;
             ++gc.n;
-            cl_blocks += c->n_samples * b->dev.NPAIR * b->dev.n_acu;
-            const int t = cluster_threads_of(b);
-            if (t > cl_threads) cl_threads = t;
-            if (cluster_smem_bytes_for(c->L) > cl_smem) cl_smem = cluster_smem_bytes_for(c->L);
+            cl_blocks += cluster_blocks_for(c->L, c->n_samples * b->dev.NPAIR * b->dev.n_acu, cl_threads);
+            if (cluster_smem_bytes_for(c->L, cl_threads) > cl_smem) cl_smem = cluster_smem_bytes_for(c->L, cl_threads);
         }
         gw.b[gw.n] = b->dev;
         gw.flags[gw.n] = PTHR_SWAP_PT | (c->er_on ? PTHR_SWAP_ER : 0);

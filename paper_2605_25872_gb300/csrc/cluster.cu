@@ -1,23 +1,38 @@
 // cluster.cu -- step (ii) of the EMCS (Sec. 3): the all-cluster Houdayer
-// update (ACU) and the original single-cluster Houdayer move, one block per
-// replica pair at one temperature.
+// update (ACU) and the original single-cluster Houdayer move.
 //
-// The block copies the two clones into shared memory and computes the site
-// overlaps q_i = s^a_i s^b_i (Eq. (2)) with one XOR per 4-site word.  It then
-// labels the connected components of {i ~ j : neighbours, q_i = q_j}:
-//  1. runs of equal q along each x row (with the periodic wrap) become stars
-//     rooted at their smallest site;
-//  2. a lock-free union-find in shared memory joins runs across y and z
-//     edges, always hooking the larger root under the smaller one, so every
-//     root is the smallest site index of its cluster (the canonical label).
-//     An edge whose left neighbours in both rows are in the same two runs is
-//     implied by that neighbouring edge and skipped; x = 0 never skips.
-// The q values of a row are one bit mask, so runs and the edges to join come
-// from a few bit operations per row.  One sign per root is drawn from Philox
-// keyed by the label; both clones flip word by word, the energies are updated
-// (on the coupling grid H_a is recomputed and H_b follows from the conserved
-// H_a + H_b) and the pair is written back.  Every loop is bounded; hitting a bound sets STATUS_NOCONVERGE
-// instead of spinning.
+// One replica pair at one temperature belongs to a group of LN lanes of a
+// warp (LN = 4, 8, 16 or 32 lanes, the smallest that holds L): lane = y, and
+// the rows z = 0..L-1 of that y sit in the lane's registers as L-bit masks
+// (bit x).  The site overlaps q_i = s^a_i s^b_i (Eq. (2)) are one XOR per
+// row.  The clusters -- connected components of {i ~ j : neighbours,
+// q_i = q_j} -- are flooded as bit masks:
+//  1. sites with no equal neighbour are clusters of their own; they drop out
+//     in one pass of bit operations over all rows;
+//  2. the first unlabelled site in site order is the next cluster's canonical
+//     label (its smallest site).  Its cluster grows from that site: a row
+//     takes in what its y and z neighbours hold, and a carry through the row's
+//     mask (m + s, and the same on the reversed row) fills whole runs along x,
+//     until a pass changes nothing.  For L <= 16 one cluster of each sign of q
+//     floods at a time, in the two halves of a word.
+// A thermalised pair (L = 12 to 16) has one large cluster of each sign, which
+// take about ten passes, and one to three others of more than one site.  A
+// pair that needs more than MAX_FLOODS turns (an overlap of hundreds of small
+// domains) is relabelled by the whole block with a union-find over its sites,
+// whose cost does not depend on the number of clusters.
+// One sign per cluster is drawn from Philox keyed by the label; the flips are
+// XORed into both clones' words and the energies are updated (on the coupling
+// grid from the bonds that the flips cut or spare, whichever are fewer, H_b
+// following from the conserved H_a + H_b).  Every loop is bounded; hitting a
+// bound sets STATUS_NOCONVERGE and leaves the pair as it was.
+//
+// What bounds it: instruction issue and latency of the floods' serial chains
+// (40% issue active, DRAM below 10%); it reads and writes each clone once.
+// Whole launch, thermalised, against the block-per-pair union-find over sites
+// that it replaces: L = 12, 28672 pairs 203 us (611 us); L = 16, 18432 pairs
+// 247 us (887 us); L = 8, 5120 pairs 36 us (44 us); at a random start, where
+// clusters are many, 269 us (705 us) and 356 us (1000 us).  Launches of few
+// pairs last as long as one warp's chain: L = 14, 840 pairs 45 us (49 us).
 #include "kernels.cuh"
 #include "bitrows.cuh"
 
@@ -25,16 +40,46 @@ namespace pthr {
 
 namespace {
 
-__device__ __forceinline__ int find_root(volatile int *parent, int x, int cap, bool &ok,
-                                         uint32_t *status = nullptr, int V = 0) {
+constexpr int MAX_FLOODS = 64;   // turns of flooding per pair before the union-find takes over
+
+template <int L>
+struct ClusterGeom {
+    static constexpr int LN = L <= 4 ? 4 : (L <= 8 ? 8 : (L <= 16 ? 16 : 32));   // lanes per pair
+    static constexpr int PPW = 32 / LN;                                          // pairs per warp
+};
+template <bool WIDE> struct RowType { typedef uint16_t T; };
+template <> struct RowType<true> { typedef uint32_t T; };
+
+// A list of bonds of one pair: site, direction (2 bits), sign (1 bit).
+template <int L>
+struct BondList {
+    static constexpr int SITE_BITS = L <= 16 ? 12 : 14;
+    typedef typename RowType<(L > 16)>::T Entry;         // 15 or 17 bits
+    static constexpr int N = 3 * L * L + L * L / 2;      // entries
+};
+
+// Shared memory: three row arrays and a bond list per pair of the block, then
+// the union-find's parents [V] and sizes [V], 16 bits each (V <= 24^3), and
+// the pairs' records.
+template <int L>
+constexpr size_t cluster_smem(int threads) {
+    typedef typename RowType<(L > 16)>::T Row;
+    const size_t slots = (size_t)(threads / 32) * ClusterGeom<L>::PPW;
+    const size_t rows = slots * (3 * L * L + BondList<L>::N) * sizeof(Row);
+    return ((rows + 15) & ~(size_t)15) + 2 * (((size_t)L * L * L * 2 + 15) & ~(size_t)15) + slots * 7 * sizeof(int);
+}
+
+// ------------------------------------------------------------ union-find
+__device__ __forceinline__ int find_root(volatile uint16_t *parent, int x, int cap, bool &ok,
+                                         uint32_t *status, int V) {
     for (int it = 0; it < cap; ++it) {
         const int p = parent[x];
         if (p == x) return x;
 #ifdef PTHR_DEBUG
-        if (!PTHR_DCHECK(status, p >= 0 && p < V && parent[p] >= 0 && parent[p] < V)) { ok = false; return x; }
+        if (!PTHR_DCHECK(status, p >= 0 && p < V && parent[p] < V)) { ok = false; return x; }
 #endif
         const int gp = parent[p];
-        if (gp != p) parent[x] = gp;   // path halving: gp is an ancestor of x
+        if (gp != p) parent[x] = (uint16_t)gp;   // path halving: gp is an ancestor of x
         x = gp;
     }
     ok = false;
@@ -45,8 +90,8 @@ __device__ __forceinline__ int find_root(volatile int *parent, int x, int cap, b
 // is done: the forest no longer changes, but other threads are writing the
 // final roots, and a path-halving store could replace a final root with an
 // intermediate ancestor after its owner wrote it.
-__device__ __forceinline__ int find_root_readonly(volatile int *parent, int x, int cap, bool &ok,
-                                                  uint32_t *status = nullptr, int V = 0) {
+__device__ __forceinline__ int find_root_readonly(volatile uint16_t *parent, int x, int cap, bool &ok,
+                                                  uint32_t *status, int V) {
     for (int it = 0; it < cap; ++it) {
         const int p = parent[x];
         if (p == x) return x;
@@ -59,195 +104,117 @@ __device__ __forceinline__ int find_root_readonly(volatile int *parent, int x, i
     return x;
 }
 
-__device__ __forceinline__ void unite(volatile int *parent, int a, int b, int cap, bool &ok,
-                                      uint32_t *status = nullptr, int V = 0) {
+__device__ __forceinline__ void unite(volatile uint16_t *parent, int a, int b, int cap, bool &ok,
+                                      uint32_t *status, int V) {
     for (int it = 0; it < cap; ++it) {
         a = find_root(parent, a, cap, ok, status, V);
         b = find_root(parent, b, cap, ok, status, V);
         if (!ok || a == b) return;
         if (a < b) { const int t = a; a = b; b = t; }   // hook the larger root a under b
-        const int old = atomicCAS(const_cast<int *>(&parent[a]), a, b);
-        if (old == a) return;
+        const unsigned short old = atomicCAS(const_cast<unsigned short *>((volatile unsigned short *)&parent[a]),
+                                             (unsigned short)a, (unsigned short)b);
+        if (old == (unsigned short)a) return;
     }
     ok = false;
 }
 
-// compact_bits, spread_bits and rot_next: bitrows.cuh; sign_nibble: pthr_internal.cuh
+struct PairStats { int nclus, top1, top2; };
 
-// natural site index of byte kk of packed word w
-template <int L>
-__device__ __forceinline__ int site_of_word(int w, int kk) {
-    using Gm = Geom<L>;
-    constexpr int W = Gm::W, ROWS = Gm::ROWS;
-    const int c = w / (ROWS * W);
-    const int g = w - c * ROWS * W;
-    const int r = g / W, j = g - (g / W) * W;
-    const int y = r % L, z = r / L;
-    const int x = 2 * (4 * j + kk) + ((c + y + z) & 1);
-    return x + L * r;
+__device__ __forceinline__ void add_size(PairStats &s, int c) {
+    ++s.nclus;
+    if (c > s.top1) { s.top2 = s.top1; s.top1 = c; } else if (c > s.top2) { s.top2 = c; }
 }
 
-// FP32 TwoSum pair (h, l) of this thread's share of sum_i sum_mu J_{i,mu}
-// s_i s_{i+mu} over the forward bonds of clone S (packed layout).  Every term
-// +-J is exact; h + l is the exact sum while l does not round.
-// With S2 set, the same for a second clone into (*h2, *l2) in the same pass.
-template <int L>
-__device__ __forceinline__ void clone_energy_pairs(const uint32_t *S, const float *J, int tid, int T,
-                                                   float &h, float &l, const uint32_t *S2 = nullptr,
-                                                   float *h2 = nullptr, float *l2 = nullptr) {
-    using Gm = Geom<L>;
-    constexpr int V = Gm::V, LW = Gm::LAT_WORDS, W = Gm::W, Lh = Gm::Lh;
-    for (int w = tid; w < LW; w += T) {
-        const int c = w / (Gm::ROWS * W);
-        const int g = w - c * Gm::ROWS * W;
-        const GroupGeo q = group_geo<L>(g, c);
-        const int j = g % W;
-        const uint32_t X = 0x3F3F3F3Fu;
-        const uint32_t o = S[q.own];
-        const uint32_t x = q.par ? __byte_perm(S[q.wA], S[q.wB], q.selx) : S[q.xa];
-        // bytes 0x3F where s_i s_{i+mu} = +1, 0xBF where -1
-        const uint32_t px = o ^ x ^ X, py = o ^ S[q.yp] ^ X, pz = o ^ S[q.zp] ^ X;
-        uint32_t px2 = 0, py2 = 0, pz2 = 0;
-        if (S2) {
-            const uint32_t o2 = S2[q.own];
-            const uint32_t x2 = q.par ? __byte_perm(S2[q.wA], S2[q.wB], q.selx) : S2[q.xa];
-            px2 = o2 ^ x2 ^ X;
-            py2 = o2 ^ S2[q.yp] ^ X;
-            pz2 = o2 ^ S2[q.zp] ^ X;
-        }
-#pragma unroll
-        for (int kk = 0; kk < 4; ++kk) {
-            if (!Gm::FULL && 4 * j + kk >= Lh) continue;
-            const int i = site_of_word<L>(w, kk);
-            const float Jx = J[i], Jy = J[V + i], Jz = J[2 * V + i];
-            two_sum_acc(h, l, Jx * spinf(px, kk));
-            two_sum_acc(h, l, Jy * spinf(py, kk));
-            two_sum_acc(h, l, Jz * spinf(pz, kk));
-            if (S2) {
-                two_sum_acc(*h2, *l2, Jx * spinf(px2, kk));
-                two_sum_acc(*h2, *l2, Jy * spinf(py2, kk));
-                two_sum_acc(*h2, *l2, Jz * spinf(pz2, kk));
-            }
-        }
-    }
+// ------------------------------------------------------------ rows
+// Rows whose words are loaded together (a divisor of L)
+__host__ __device__ constexpr int rows_in_flight(int L) {
+    const int most = L > 16 ? 4 : 8;
+    for (int n = most; n > 1; --n)
+        if (L % n == 0) return n;
+    return 1;
 }
 
-// CAPPED = false: every loop bound is the compile-time constant 4V+64 (the
-// production path; a runtime bound makes the labelling loops markedly
-// slower).  CAPPED = true: the bound comes from the tuning knob, used only to
-// exercise the error path.
-template <int L, bool CAPPED>
-__device__ __forceinline__ void cluster_block(const ClusterArgs &a, int bid, unsigned char *smem) {
-    using Gm = Geom<L>;
-    constexpr int V = Gm::V, LW = Gm::LAT_WORDS, W = Gm::W, Lh = Gm::Lh;
-    int *parent = reinterpret_cast<int *>(smem);                       // [V]
-    int *cnt = parent + V;                                             // [V]
-    uint32_t *sa = reinterpret_cast<uint32_t *>(cnt + V);              // [LW]
-    uint32_t *sb = sa + LW;                                            // [LW]
-    unsigned char *flag = reinterpret_cast<unsigned char *>(sb + LW);  // [V] sign of each root
-    uint32_t *qrow = reinterpret_cast<uint32_t *>(flag + ((V + 3) & ~3));  // [L*L] q bits per x row,
-                                                                           // later the flip bits
-    uint32_t *arow = qrow + L * L;                                     // [L*L] clone a: 1 = spin -1
-    int *s_scan = reinterpret_cast<int *>(arow + L * L);               // [blockDim.x] row-count scan
-    __shared__ int s_ok;
-    __shared__ int s_nneg, s_root, s_nclus, s_nflip;
-    __shared__ int s_top[2][32];
-    __shared__ double s_E[2];
-    __shared__ unsigned long long s_Ei[1];
+// flip mask of packed word j (bit 7 of byte k: site 4j + k of the colour
+// row) from the natural row's flip bits shifted to the colour's parity
+__device__ __forceinline__ uint32_t word_flips(uint32_t v, int j) {
+    return (((v >> (8 * j)) & 0x55u) * 0x02082080u) & 0x80808080u;
+}
 
+// ------------------------------------------------------------ items
+struct PairItem {
+    bool live;
+    int s, P, k, la, lb;
+    uint32_t emcs, pair_id;
+    unsigned long long seed;
+};
+
+__device__ __forceinline__ PairItem pair_item(const ClusterArgs &a, int item) {
     const Batch &b = a.b;
-    const int n_acu = b.n_acu;
-    int t = bid;
-    const int k = t % n_acu; t /= n_acu;
-    const int P = t % b.NPAIR; t /= b.NPAIR;
-    const int s = a.sample_first + t;
-    if (!PTHR_DCHECK(b.status, s >= 0 && s < b.S && k < b.NT && P < b.NPAIR)) return;
-    if (!b.active[s]) return;
-    const uint32_t emcs = b.emcs[s];
-    if (!a.label_only && (emcs % (uint32_t)b.acu_interval) != 0u) return;
-    const unsigned long long seed = b.seeds[s];
-    const int tid = threadIdx.x, T = blockDim.x;
-    const int ga = 2 * P, gb = 2 * P + 1;
-    const int la = ga * b.NSLOT + b.perm[((size_t)s * b.NR + ga) * b.NSLOT + k];
-    const int lb = gb * b.NSLOT + b.perm[((size_t)s * b.NR + gb) * b.NSLOT + k];
-    if (!PTHR_DCHECK(b.status, la >= ga * b.NSLOT && la < (ga + 1) * b.NSLOT &&
-                                lb >= gb * b.NSLOT && lb < (gb + 1) * b.NSLOT && gb < b.NR)) return;
-    const uint32_t pair_id = (uint32_t)(P * b.NT + k);
-    uint32_t *ga_ptr = b.spins + ((size_t)s * b.NLAT + la) * b.lat_words;
-    uint32_t *gb_ptr = b.spins + ((size_t)s * b.NLAT + lb) * b.lat_words;
-    constexpr int LB8 = LW / 8;     // bit words per lattice (bit storage)
+    PairItem p{};
+    if (item >= a.sample_count * b.NPAIR * b.n_acu) return p;
+    int t = item;
+    p.k = t % b.n_acu; t /= b.n_acu;
+    p.P = t % b.NPAIR; t /= b.NPAIR;
+    p.s = a.sample_first + t;
+    if (!PTHR_DCHECK(b.status, p.s >= 0 && p.s < b.S && p.k < b.NT && p.P < b.NPAIR)) return PairItem{};
+    if (!b.active[p.s]) return p;
+    p.emcs = b.emcs[p.s];
+    if (!a.label_only && (p.emcs % (uint32_t)b.acu_interval) != 0u) return p;
+    p.seed = b.seeds[p.s];
+    const int ga = 2 * p.P, gb = 2 * p.P + 1;
+    p.la = ga * b.NSLOT + b.perm[((size_t)p.s * b.NR + ga) * b.NSLOT + p.k];
+    p.lb = gb * b.NSLOT + b.perm[((size_t)p.s * b.NR + gb) * b.NSLOT + p.k];
+    if (!PTHR_DCHECK(b.status, p.la >= ga * b.NSLOT && p.la < (ga + 1) * b.NSLOT &&
+                                p.lb >= gb * b.NSLOT && p.lb < (gb + 1) * b.NSLOT && gb < b.NR)) return PairItem{};
+    p.pair_id = (uint32_t)(p.P * b.NT + p.k);
+    p.live = true;
+    return p;
+}
 
-    if (tid == 0) { s_ok = 1; s_nneg = 0; s_root = -1; s_nclus = 0; s_nflip = 0; }
-    if (tid < 2) s_E[tid] = 0.0;
-    if (tid == 0) s_Ei[0] = 0ull;
-    if (b.bits) {
-        for (int i = tid; i < 2 * LB8; i += T) {
-            const int u = i < LB8 ? i : i - LB8;
-            uint4 lo, hi;
-            expand_bits(i < LB8 ? ga_ptr[u] : gb_ptr[u], lo, hi);
-            uint4 *d = reinterpret_cast<uint4 *>((i < LB8 ? sa : sb) + 8 * u);
-            d[0] = lo;
-            d[1] = hi;
-        }
-    } else {
-        for (int i = tid; i < LW / 4; i += T) {
-            reinterpret_cast<uint4 *>(sa)[i] = reinterpret_cast<const uint4 *>(ga_ptr)[i];
-            reinterpret_cast<uint4 *>(sb)[i] = reinterpret_cast<const uint4 *>(gb_ptr)[i];
-        }
-    }
-    __syncthreads();
-    // q bits of every natural x row r = y + L z: bit x of qrow[r] is 1 iff
-    // q_i = -1 at i = x + L r.  The two clones' bytes differ exactly there
-    // (0x3F vs 0xBF): one XOR per 4 sites, a multiply gathers the four sign
-    // bits, and the two colour rows interleave (colour c holds x = 2m + p_c).
-    constexpr uint32_t M = L == 32 ? 0xffffffffu : ((1u << L) - 1u);
-    for (int r = tid; r < L * L; r += T) {
-        const int y = r % L, z = r / L;
-        uint32_t bits[2], abits[2];
-#pragma unroll
-        for (int c = 0; c < 2; ++c) {
-            uint32_t acc = 0, aacc = 0;
-#pragma unroll
-            for (int j = 0; j < W; ++j) {
-                const int w = (c * Gm::ROWS + r) * W + j;
-                acc |= sign_nibble(sa[w] ^ sb[w]) << (4 * j);
-                aacc |= sign_nibble(sa[w]) << (4 * j);
-            }
-            bits[c] = acc & ((1u << Lh) - 1u);
-            abits[c] = aacc & ((1u << Lh) - 1u);
-        }
-        const int p0 = (y + z) & 1;
-        qrow[r] = (spread_bits(bits[0]) << p0) | (spread_bits(bits[1]) << (p0 ^ 1));
-        arow[r] = (spread_bits(abits[0]) << p0) | (spread_bits(abits[1]) << (p0 ^ 1));
-    }
-    for (int i = tid; i < V; i += T) cnt[i] = 0;
-    __syncthreads();
-    // 1. runs of equal q along each periodic x row, rooted at their first
-    //    site; the last run is rooted at x = 0 when it wraps onto the first
+// eta = -1 iff the top bit of word 0 of (label, pair_id, emcs, TAG_ACU)
+__device__ __forceinline__ bool cluster_sign(const PairItem &p, int label) {
+    return (philox_word0(p.seed, (uint32_t)label, p.pair_id, p.emcs, TAG_ACU) >> 31) != 0u;
+}
+
+// Labels, flips and sizes of one pair of the block by union-find over its
+// sites (all threads of the block).  Fs receives the flip rows.
+//  1. runs of equal q along each x row (with the periodic wrap) become stars
+//     rooted at their smallest site;
+//  2. a lock-free union-find in shared memory joins runs across y and z
+//     edges, always hooking the larger root under the smaller one, so every
+//     root is the smallest site index of its cluster (the canonical label).
+//     An edge whose left neighbours in both rows are in the same two runs is
+//     implied by that neighbouring edge and skipped; x = 0 never skips.
+template <int L, typename Row>
+__device__ __noinline__ bool union_find_pair(const ClusterArgs &a, const PairItem &p, int target, const Row *qs,
+                                             Row *Fs, uint16_t *parent, uint16_t *cnt, int cap, PairStats &st) {
+    constexpr int V = L * L * L;
+    constexpr uint32_t M = (1u << L) - 1u;
+    __shared__ int s_ok, s_nclus, s_top[2][32];
+    const Batch &b = a.b;
+    const int tid = threadIdx.x, T = blockDim.x;
+    if (tid == 0) { s_ok = 1; s_nclus = 0; }
+    for (int i = tid; i < (V + 1) / 2; i += T) reinterpret_cast<uint32_t *>(cnt)[i] = 0u;
     for (int r = tid; r < L * L; r += T) {
         const int i0 = L * r;
-        const uint32_t q = qrow[r];
-        const uint32_t st = (q ^ (q << 1)) & M & ~1u;       // bit x >= 1: q[x] != q[x-1]
-        const bool wrap = ((q ^ (q >> (L - 1))) & 1u) == 0u;  // q[0] == q[L-1]
-        const int last = st ? 31 - __clz(st) : L;            // start of the last run
+        const uint32_t q = qs[r];
+        const uint32_t st_ = (q ^ (q << 1)) & M & ~1u;         // bit x >= 1: q[x] != q[x-1]
+        const bool wrap = ((q ^ (q >> (L - 1))) & 1u) == 0u;   // q[0] == q[L-1]
+        const int last = st_ ? 31 - __clz(st_) : L;            // start of the last run
         int root = i0;
         for (int x = 0; x < L; ++x) {
-            if ((st >> x) & 1u) root = i0 + x;
-            parent[i0 + x] = (wrap && x >= last) ? i0 : root;
+            if ((st_ >> x) & 1u) root = i0 + x;
+            parent[i0 + x] = (uint16_t)((wrap && x >= last) ? i0 : root);
         }
     }
     __syncthreads();
-    // 2. join runs across y and z edges, one thread per (row, direction).
-    //    Edges join equal q; an edge at x != 0 where no run starts in either
-    //    row is implied by the edge at x - 1 and skipped.
     bool ok = true;
-    const int cap = CAPPED ? a.iter_cap : 4 * V + 64;
-    volatile int *vp = parent;
+    volatile uint16_t *vp = parent;
     for (int tsk = tid; tsk < 2 * L * L; tsk += T) {
         const int r = tsk >> 1;
         const int y = r % L, z = r / L;
         const int r2 = (tsk & 1) ? y + L * ((z + 1) % L) : ((y + 1) % L) + L * z;
-        const uint32_t q1 = qrow[r], q2 = qrow[r2];
+        const uint32_t q1 = qs[r], q2 = qs[r2];
         uint32_t C = ~(q1 ^ q2) & M & ((q1 ^ (q1 << 1)) | (q2 ^ (q2 << 1)) | 1u);
         while (C) {
             const int x = __ffs(C) - 1;
@@ -258,101 +225,30 @@ __device__ __forceinline__ void cluster_block(const ClusterArgs &a, int bid, uns
     __syncthreads();
     // every site points straight at its root; only final roots are written
     // here (no path halving), so after the barrier parent[i] is the root
-    for (int i = tid; i < V; i += T) {
-        const int r = find_root_readonly(vp, i, cap, ok, b.status, V);
-        parent[i] = r;
-    }
+    for (int i = tid; i < V; i += T) parent[i] = (uint16_t)find_root_readonly(vp, i, cap, ok, b.status, V);
     if (!ok) s_ok = 0;
     __syncthreads();
-    if (!s_ok) {
-        if (tid == 0) set_status(b.status, STATUS_NOCONVERGE);
-        return;
-    }
-    if (a.labels_out) {
-        int32_t *out = a.labels_out + ((size_t)(s * b.NPAIR + P) * b.NT + k) * V;
+    if (!s_ok) return false;
+    if (a.label_only) {
+        int32_t *out = a.labels_out + ((size_t)(p.s * b.NPAIR + p.P) * b.NT + p.k) * V;
         for (int i = tid; i < V; i += T) out[i] = parent[i];
+        __syncthreads();
+        return true;
     }
     // cluster sizes (statistics): one atomic per distinct root per warp
     for (int i0 = 0; i0 < V; i0 += T) {
         const int i = i0 + tid;
         const int root = i < V ? parent[i] : -1;
         const unsigned peers = __match_any_sync(0xffffffffu, root);
-        if (i < V && (tid & 31) == __ffs(peers) - 1) atomicAdd(&cnt[root], __popc(peers));
+        if (i < V && (tid & 31) == __ffs(peers) - 1)
+            atomicAdd(reinterpret_cast<uint32_t *>(cnt) + (root >> 1), (uint32_t)__popc(peers) << (16 * (root & 1)));
     }
     __syncthreads();
-    if (a.label_only) return;
-
-    if (b.cluster_mode == PTHR_CLUSTER_ACU) {
-        // one sign per cluster: eta = -1 iff top bit of word 0 of
-        // (label, pair_id, emcs, TAG_ACU); the root's flag byte receives it
-        for (int i = tid; i < V; i += T) {
-            if (parent[i] == i) {
-                const uint32_t w = philox_word0(seed, (uint32_t)i, pair_id, emcs, TAG_ACU);
-                flag[i] = (unsigned char)(w >> 31);
-            }
-        }
-        __syncthreads();
-    } else {
-        // single cluster: seed = the floor(u*n)-th q = -1 site (natural
-        // order), n = #(q = -1); each thread counts a contiguous range of rows
-        const int chunk = (L * L + T - 1) / T;
-        const int lo = min(L * L, tid * chunk), hi = min(L * L, lo + chunk);
-        int my = 0;
-        for (int r = lo; r < hi; ++r) my += __popc(qrow[r]);
-        s_scan[tid] = my;
-        __syncthreads();
-        if (tid == 0) {
-            int acc = 0;
-            for (int u = 0; u < T; ++u) { const int v = s_scan[u]; s_scan[u] = acc; acc += v; }
-            s_nneg = acc;
-        }
-        __syncthreads();
-        const int n = s_nneg;
-        if (n > 0) {
-            const uint32_t w = philox_word0(seed, 0u, pair_id, emcs, TAG_SINGLE);
-            const int target = (int)(((unsigned long long)(w >> 8) * (unsigned long long)n) >> 24);
-            int seen = s_scan[tid];
-            if (target >= seen && target < seen + my) {
-                for (int r = lo; r < hi; ++r) {
-                    uint32_t v = qrow[r];
-                    const int c = __popc(v);
-                    if (target < seen + c) {
-                        for (int m = target - seen; m > 0; --m) v &= v - 1u;
-                        s_root = parent[L * r + __ffs(v) - 1];
-                        break;
-                    }
-                    seen += c;
-                }
-            }
-        }
-        __syncthreads();
-        const int root = s_root;
-        for (int i = tid; i < V; i += T)
-            if (parent[i] == i) flag[i] = (unsigned char)(i == root);
-        __syncthreads();
-    }
-    // flip bits of every natural x row (bit x set iff the cluster of site
-    // x + L r is flipped); the q rows are no longer needed
-    uint32_t *frow = qrow;
-    int nflip = 0;
-    for (int r = tid; r < L * L; r += T) {
-        uint32_t f = 0u;
-#pragma unroll
-        for (int x = 0; x < L; ++x) f |= (uint32_t)flag[parent[L * r + x]] << x;
-        frow[r] = f;
-        nflip += __popc(f);
-    }
-    // statistics: number of clusters, two largest sizes
-    int nroots = 0, t1 = 0, t2 = 0;
-    for (int i = tid; i < V; i += T) {
-        if (parent[i] == i) {
-            ++nroots;
-            const int c = cnt[i];
-            if (c > t1) { t2 = t1; t1 = c; } else if (c > t2) { t2 = c; }
-        }
-    }
-    atomicAdd(&s_nclus, nroots);
-    atomicAdd(&s_nflip, nflip);
+    PairStats my{0, 0, 0};
+    for (int i = tid; i < V; i += T)
+        if (parent[i] == i) add_size(my, cnt[i]);
+    atomicAdd(&s_nclus, my.nclus);
+    int t1 = my.top1, t2 = my.top2;
     for (int o = 16; o > 0; o >>= 1) {
         const int u1 = __shfl_xor_sync(0xffffffffu, t1, o), u2 = __shfl_xor_sync(0xffffffffu, t2, o);
         int n1, n2;
@@ -361,140 +257,642 @@ __device__ __forceinline__ void cluster_block(const ClusterArgs &a, int bid, uns
     }
     if ((tid & 31) == 0) { s_top[0][tid >> 5] = t1; s_top[1][tid >> 5] = t2; }
     __syncthreads();
-    // flip both clones word by word: the colour-c bits of the row mask,
-    // compacted, give the word's four flip bits
-    for (int w = tid; w < LW; w += T) {
-        const int c = w / (Gm::ROWS * W);
-        const int g = w - c * Gm::ROWS * W;
-        const int r = g / W, j = g - r * W;
-        const int y = r % L, z = r / L;
-        const uint32_t nib = (compact_bits(frow[r] >> ((c + y + z) & 1)) >> (4 * j)) & 0xFu;
-        const uint32_t m = ((nib * 0x00204081u) & 0x01010101u) << 7;
-        sa[w] ^= m;
-        sb[w] ^= m;
+    // the sizes are read: a root's entry now holds its flip bit
+    const int root_t = target >= 0 ? parent[target] : -1;
+    for (int i = tid; i < V; i += T)
+        if (parent[i] == i)
+            cnt[i] = (uint16_t)(b.cluster_mode == PTHR_CLUSTER_ACU ? cluster_sign(p, i) : i == root_t);
+    int a1 = 0, a2 = 0;
+    for (int w = 0; w < T / 32; ++w) {
+        const int u1 = s_top[0][w], u2 = s_top[1][w];
+        if (u1 > a1) { a2 = max(a1, u2); a1 = u1; } else { a2 = max(a2, u1); }
     }
-    // energies (Eq. (1)).  Only bonds with exactly one flipped end change:
+    st = PairStats{s_nclus, a1, a2};
+    __syncthreads();
+    for (int r = tid; r < L * L; r += T) {
+        uint32_t f = 0u;
+        for (int x = 0; x < L; ++x) f |= (uint32_t)cnt[parent[L * r + x]] << x;
+        Fs[r] = (Row)f;
+    }
+    __syncthreads();
+    return true;
+}
+
+// A lane's rows hold the unlabelled sites of both signs of q: for L <= 16 the
+// q = +1 sites in the low and the q = -1 sites in the high half of one word,
+// so that one cluster of each sign floods at a time; for larger L two words.
+template <int L>
+struct FloodWords {
+    static constexpr bool PACKED = L <= 16;
+    static constexpr uint32_t M = (1u << L) - 1u;
+    // bits of the row's first and last site, in both halves
+    static constexpr uint32_t FIRST = PACKED ? 0x00010001u : 1u;
+    static constexpr uint32_t LAST = FIRST << (L - 1);
+};
+
+// a + b, by halves where the row fills a half (otherwise a carry out of the
+// low row ends in the gap above it, which no mask holds)
+template <int L>
+__device__ __forceinline__ uint32_t add_rows(uint32_t a, uint32_t b) {
+    if (L != 16) return a + b;
+    uint32_t d;
+    asm("add.u16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
+    return d;
+}
+
+// One row of a flood: row z takes in what its neighbour rows hold and fills
+// whole runs of its mask m (mr: reversed).  The carries of m + s run from a
+// seed to its run's top, on the reversed row to its bottom.  Returns the new
+// bits.
+template <int L>
+__device__ __forceinline__ uint32_t flood_row(uint32_t (&f)[L], const uint32_t (&m)[L], const uint32_t (&mr)[L],
+                                              int z, int lp, int lm) {
+    using Fw = FloodWords<L>;
+    const uint32_t f0 = f[z];
+    const uint32_t fy = __shfl_sync(0xffffffffu, f0, lp) | __shfl_sync(0xffffffffu, f0, lm);
+    uint32_t s = f0 | f[(z + 1) % L] | f[(z + L - 1) % L];
+    s = s | fy | ((f0 >> (L - 1)) & Fw::FIRST);
+    s = (s | ((f0 << (L - 1)) & Fw::LAST)) & m[z];
+    const uint32_t sr = __brev(s);
+    const uint32_t up = (m[z] & ~add_rows<L>(m[z], s)) | s;
+    const uint32_t dn = (mr[z] & ~add_rows<L>(mr[z], sr)) | sr;
+    f[z] = up | __brev(dn);
+    return f[z] ^ f0;
+}
+
+// Energies, flips and statistics of the pairs of a warp, from their flip rows.
+template <int L, typename Row>
+__device__ __forceinline__ void finish_pair(const ClusterArgs &a, const PairItem &p, const Row *qs, const Row *as,
+                                         const Row *Fs, typename BondList<L>::Entry *list, int *count, int sub, int yl, bool ok,
+                                            bool rest, const PairStats &st) {
+    using Gm = Geom<L>;
+    constexpr int V = Gm::V, LW = Gm::LAT_WORDS, W = Gm::W, ROWS = Gm::ROWS;
+    constexpr int LN = ClusterGeom<L>::LN, SITE_BITS = BondList<L>::SITE_BITS;
+    constexpr unsigned FULLW = 0xffffffffu;
+    typedef typename BondList<L>::Entry Entry;
+    const Batch &b = a.b;
+    const int y = yl < L ? yl : L - 1, yp = (y + 1) % L;
+    uint32_t *A = b.spins + ((size_t)p.s * b.NLAT + p.la) * b.lat_words;
+    uint32_t *B = b.spins + ((size_t)p.s * b.NLAT + p.lb) * b.lat_words;
+    if (p.live && !ok && yl == 0) set_status(b.status, STATUS_NOCONVERGE);
+    __syncwarp();
+    if (a.label_only) return;
+    const bool go = p.live && ok;                        // the same for all lanes of the pair
+
+    // ---- energies (Eq. (1)).  Only bonds with exactly one flipped end change:
     // for them s'_i s'_j = -s_i s_j, so Delta H_a = sum of 2 J s_i s_j (old
     // spins of clone a).  Such a bond joins sites of opposite q, where the two
     // clones' terms cancel, so H_a + H_b is conserved and Delta H_b =
-    // -Delta H_a.  On the coupling grid (every thread's FP32 pair sum a
-    // multiple of 2^-18) Delta H_a is summed exactly in integers and both
-    // energies are updated exactly in FP64; the energies before are those of
-    // the resident spins (every entry point that changes spins recomputes
-    // them).  Off the grid both energies are recomputed and reduced in FP64.
-    const float *J = b.J + (size_t)s * 3 * V;
-    float ha = 0.f, la_ = 0.f;
-    for (int r = tid; r < L * L; r += T) {
-        const int y = r % L, z = r / L;
-        const int ry = ((y + 1) % L) + L * z, rz = y + L * ((z + 1) % L);
-        const uint32_t f = frow[r], av = arow[r];
-        const uint32_t cut[3] = {f ^ rot_next<L>(f), f ^ frow[ry], f ^ frow[rz]};
-        const uint32_t neg[3] = {av ^ rot_next<L>(av), av ^ arow[ry], av ^ arow[rz]};
+    // -Delta H_a.  Over all bonds between opposite q the same sum is
+    // H_b - H_a, so with R the sum over those that are NOT cut, the new
+    // energies are H_b - R and H_a + R.  `rest` picks the shorter sum: when
+    // the two large clusters (one of each sign) flip differently, nearly
+    // every bond between them is cut and R runs over the bonds at small
+    // clusters only, and when they flip alike the cut bonds do (a thermalised
+    // pair has 30% of its bonds between opposite q and cuts none or nearly
+    // all of them; either sum then has a few dozen terms).
+    // On the coupling grid (J a multiple of 2^-18) the sum is exact in
+    // integers and both energies are updated exactly in FP64; the energies
+    // before are those of the resident spins (every entry point that changes
+    // spins recomputes them).  Off the grid both energies are recomputed.
+    const float *J = b.J + (size_t)p.s * 3 * V;
+    long long dE = 0;
+    int nflip = 0;
+    uint32_t bad = 0;                                    // a coupling off the grid
+    // The bonds go through a list in shared memory (site, direction and the
+    // sign of s_i s_j in one entry): the lanes' rows hold very different
+    // numbers of them, and from the list every lane sums an equal share with
+    // its couplings' loads (600 to 800 cycles each) in flight together.
+    if (yl == 0) *count = 0;
+    __syncwarp();
+    int listed = 0;                                      // entries, the same for all lanes of the pair
+    for (int z = 0; z < L; ++z) {
+        const int r = y + L * z, ry = yp + L * z, rz = y + L * (z + 1 == L ? 0 : z + 1);
+        uint32_t w[3] = {0u, 0u, 0u}, n[3];
+        if (go && yl < L) {
+            const uint32_t f = Fs[r], av = as[r];
+            nflip += __popc(f);
+            w[0] = f ^ rot_next<L>(f);
+            w[1] = f ^ Fs[ry];
+            w[2] = f ^ Fs[rz];
+            if (rest) {
+                const uint32_t q = qs[r];
+                w[0] ^= q ^ rot_next<L>(q);
+                w[1] ^= q ^ qs[ry];
+                w[2] ^= q ^ qs[rz];
+            }
+            n[0] = av ^ rot_next<L>(av);
+            n[1] = av ^ as[ry];
+            n[2] = av ^ as[rz];
+            const int mine = __popc(w[0]) + __popc(w[1]) + __popc(w[2]);
+            if (mine) {
+                int at = atomicAdd(count, mine);
 #pragma unroll
-        for (int d = 0; d < 3; ++d) {
-            uint32_t cb = cut[d];
-            while (cb) {
-                const int x = __ffs(cb) - 1;
-                cb &= cb - 1u;
-                const float t = 2.f * J[d * V + L * r + x];
-                two_sum_acc(ha, la_, ((neg[d] >> x) & 1u) ? -t : t);
+                for (int d = 0; d < 3; ++d) {
+                    while (w[d]) {
+                        const int sh = __clz(w[d]), x = 31 - sh;
+                        w[d] ^= 1u << x;
+                        list[at++] = (Entry)((L * r + x) | (d << SITE_BITS) | (((n[d] >> x) & 1u) << (SITE_BITS + 2)));
+                    }
+                }
+            }
+        }
+        __syncwarp();
+        listed = *count;
+        // a plane holds at most 3 L^2 bonds: sum the list up when the next plane
+        // may not fit (or at the end)
+        if (__any_sync(FULLW, listed > BondList<L>::N - 3 * L * L) || z == L - 1) {
+            int sum = 0;
+#pragma unroll 4
+            for (int i = yl; i < listed; i += LN) {
+                const uint32_t e = list[i];
+                const uint32_t site = e & ((1u << SITE_BITS) - 1u), d = (e >> SITE_BITS) & 3u;
+                const float j = __uint_as_float(__float_as_uint(__ldg(J + d * V + site)) ^ ((e >> (SITE_BITS + 2)) << 31));
+                // J 2^18 as an integer (adding 1.5 2^23 rounds to one); it is
+                // J exactly iff the integer gives J back bit for bit
+                const int v = __float_as_int(fmaf(j, 262144.f, 12582912.f)) - 0x4B400000;
+                bad |= __float_as_uint((float)v * 3.814697265625e-06f) ^ __float_as_uint(j);
+                sum += v;                                // at most N / LN terms below 2^23
+            }
+            dE += sum;
+            __syncwarp();
+            if (yl == 0) *count = 0;
+            __syncwarp();
+        }
+    }
+    const unsigned off = __ballot_sync(FULLW, bad != 0u);
+    const bool exact_E = ((off >> (sub * LN)) & (unsigned)((1ull << LN) - 1ull)) == 0u;
+    double Ea = 0.0, Eb = 0.0;
+    if (go && !exact_E && yl < L) {
+        float h = 0.f, l = 0.f, h2 = 0.f, l2 = 0.f;
+        for (int z = 0; z < L; ++z) {
+            const int r = y + L * z, ry = yp + L * z, rz = y + L * ((z + 1) % L);
+            const uint32_t ar = as[r] ^ Fs[r], ay = as[ry] ^ Fs[ry], az = as[rz] ^ Fs[rz];
+            const uint32_t br = ar ^ qs[r], by = ay ^ qs[ry], bz = az ^ qs[rz];
+            const uint32_t na[3] = {ar ^ rot_next<L>(ar), ar ^ ay, ar ^ az};
+            const uint32_t nb[3] = {br ^ rot_next<L>(br), br ^ by, br ^ bz};
+            for (int x = 0; x < L; ++x) {
+#pragma unroll
+                for (int d = 0; d < 3; ++d) {
+                    const float j = __ldg(J + d * V + L * r + x);
+                    two_sum_acc(h, l, ((na[d] >> x) & 1u) ? -j : j);
+                    two_sum_acc(h2, l2, ((nb[d] >> x) & 1u) ? -j : j);
+                }
+            }
+        }
+        Ea = (double)h + (double)l;
+        Eb = (double)h2 + (double)l2;
+    }
+    for (int o = LN / 2; o > 0; o >>= 1) {
+        dE += __shfl_xor_sync(FULLW, dE, o);
+        nflip += __shfl_xor_sync(FULLW, nflip, o);
+    }
+    if (off) {                                           // warp-uniform
+        for (int o = LN / 2; o > 0; o >>= 1) {
+            Ea += __shfl_xor_sync(FULLW, Ea, o);
+            Eb += __shfl_xor_sync(FULLW, Eb, o);
+        }
+    }
+    if (!go) return;
+    // ---- flip both clones
+    if (b.bits) {
+        for (int i = yl; i < LW / 8; i += LN) {
+            uint32_t m = 0;
+#pragma unroll
+            for (int t = 0; t < 8; ++t) {
+                const int w = 8 * i + t;
+                const int c = w / (ROWS * W), g = w - c * ROWS * W;
+                const int r = g / W, j = g - r * W;
+                m |= (compact_bits((uint32_t)Fs[r] >> ((c + r % L + r / L) & 1)) >> (4 * j) & 0xFu) << (4 * t);
+            }
+            if (m) { A[i] ^= m; B[i] ^= m; }
+        }
+    } else if (yl < L) {
+        // four rows at a time, so that their loads are in flight together
+        constexpr int ZB = L % 4 == 0 ? 4 : 2;
+        for (int z0 = 0; z0 < L; z0 += ZB) {
+            uint32_t f[ZB], wa[ZB][2][W], wb[ZB][2][W];
+#pragma unroll
+            for (int i = 0; i < ZB; ++i) {
+                const int r = y + L * (z0 + i);
+                f[i] = Fs[r];
+                if (f[i]) {
+#pragma unroll
+                    for (int c = 0; c < 2; ++c) {
+                        load_words<W>(A + (c * ROWS + r) * W, wa[i][c]);
+                        load_words<W>(B + (c * ROWS + r) * W, wb[i][c]);
+                    }
+                }
+            }
+#pragma unroll
+            for (int i = 0; i < ZB; ++i) {
+                const int r = y + L * (z0 + i);
+                if (!f[i]) continue;
+#pragma unroll
+                for (int c = 0; c < 2; ++c) {
+                    const uint32_t v = f[i] >> ((c + y + z0 + i) & 1);
+#pragma unroll
+                    for (int j = 0; j < W; ++j) {
+                        const uint32_t mj = word_flips(v, j);
+                        wa[i][c][j] ^= mj;
+                        wb[i][c][j] ^= mj;
+                    }
+                    store_words<W>(A + (c * ROWS + r) * W, wa[i][c]);
+                    store_words<W>(B + (c * ROWS + r) * W, wb[i][c]);
+                }
             }
         }
     }
-    const float xa = ha * 262144.f, xla = la_ * 262144.f;
-    const bool ig = xa == rintf(xa) && xla == rintf(xla) && fabsf(xa) < 536870912.f && fabsf(xla) < 65536.f;
-    const bool exact_E = __syncthreads_and(ig) != 0;
-    if (exact_E) {
-        const int va = __float2int_rn(xa) + __float2int_rn(xla);
-        // split so that the 32-lane sums cannot overflow
-        const int ah = __reduce_add_sync(0xffffffffu, va >> 12);
-        const unsigned al = __reduce_add_sync(0xffffffffu, (unsigned)(va & 0xFFF));
-        if ((tid & 31) == 0) atomicAdd(&s_Ei[0], (unsigned long long)((long long)ah * 4096 + (long long)al));
-    } else {
-        float hb = 0.f, lb_ = 0.f;
-        ha = 0.f;
-        la_ = 0.f;
-        clone_energy_pairs<L>(sa, J, tid, T, ha, la_, sb, &hb, &lb_);
-        double ea = (double)ha + (double)la_, eb = (double)hb + (double)lb_;
-        for (int o = 16; o > 0; o >>= 1) {
-            ea += __shfl_xor_sync(0xffffffffu, ea, o);
-            eb += __shfl_xor_sync(0xffffffffu, eb, o);
-        }
-        if ((tid & 31) == 0) { atomicAdd(&s_E[0], ea); atomicAdd(&s_E[1], eb); }
-    }
-    __syncthreads();
-    if (b.bits) {
-        for (int i = tid; i < 2 * LB8; i += T) {
-            const int u = i < LB8 ? i : i - LB8;
-            const uint4 *w = reinterpret_cast<const uint4 *>((i < LB8 ? sa : sb) + 8 * u);
-            (i < LB8 ? ga_ptr : gb_ptr)[u] = pack_bits(w[0], w[1]);
-        }
-    } else {
-        for (int i = tid; i < LW / 4; i += T) {
-            reinterpret_cast<uint4 *>(ga_ptr)[i] = reinterpret_cast<const uint4 *>(sa)[i];
-            reinterpret_cast<uint4 *>(gb_ptr)[i] = reinterpret_cast<const uint4 *>(sb)[i];
-        }
-    }
-    if (tid == 0) {
-        double *E = b.E + (size_t)s * b.NLAT;
+    if (yl == 0) {
+        double *E = b.E + (size_t)p.s * b.NLAT;
         if (exact_E) {
-            const double dH = (double)(long long)s_Ei[0] * (1.0 / 262144.0);
-            E[la] = E[la] + dH;
-            E[lb] = E[lb] - dH;
+            const double dH = (double)(2 * dE) * (1.0 / 262144.0);
+            const double Ha = E[p.la], Hb = E[p.lb];
+            E[p.la] = rest ? Hb - dH : Ha + dH;
+            E[p.lb] = rest ? Ha + dH : Hb - dH;
         } else {
-            E[la] = -s_E[0];
-            E[lb] = -s_E[1];
+            E[p.la] = -Ea;
+            E[p.lb] = -Eb;
         }
-        int a1 = 0, a2 = 0;
-        for (int w = 0; w < (T + 31) / 32; ++w) {
-            const int u1 = s_top[0][w], u2 = s_top[1][w];
-            if (u1 > a1) { a2 = max(a1, u2); a1 = u1; } else { a2 = max(a2, u1); }
-        }
-        long long *cs = b.cstat + (((size_t)s * b.NPAIR + P) * b.NT + k) * 4;
-        cs[0] = s_nclus;
-        cs[1] = a1;
-        cs[2] = a2;
-        cs[3] = s_nflip;
+        long long *cs = b.cstat + (((size_t)p.s * b.NPAIR + p.P) * b.NT + p.k) * 4;
+        cs[0] = st.nclus;
+        cs[1] = st.top1;
+        cs[2] = st.top2;
+        cs[3] = nflip;
     }
 }
 
-template <int L, bool CAPPED>
-__global__ void __launch_bounds__(512, 4) cluster_kernel(ClusterArgs a) {
-    extern __shared__ __align__(16) unsigned char smem[];
-    cluster_block<L, CAPPED>(a, blockIdx.x, smem);
+
+// ------------------------------------------------------------ the block
+template <int L>
+__device__ __forceinline__ void cluster_block(const ClusterArgs &a, int bid, unsigned char *smem) {
+    using Gm = Geom<L>;
+    constexpr int V = Gm::V, ROWS = Gm::ROWS, W = Gm::W;
+    constexpr int LN = ClusterGeom<L>::LN, PPW = ClusterGeom<L>::PPW;
+    constexpr uint32_t M = (1u << L) - 1u;
+    constexpr unsigned FULLW = 0xffffffffu;
+    typedef typename RowType<(L > 16)>::T Row;
+    const Batch &b = a.b;
+    const int tid = threadIdx.x, T = blockDim.x;
+    const int lane = tid & 31, sub = lane / LN, yl = lane % LN;
+    const int slots = (T / 32) * PPW, slot = (tid >> 5) * PPW + sub;
+    Row *rows = reinterpret_cast<Row *>(smem);
+    Row *qs = rows + (size_t)slot * 3 * ROWS, *as = qs + ROWS, *Fs = as + ROWS;
+    Row *list = rows + (size_t)slots * 3 * ROWS + (size_t)slot * BondList<L>::N;
+    uint16_t *parent = reinterpret_cast<uint16_t *>(
+        smem + (((size_t)slots * (3 * ROWS + BondList<L>::N) * sizeof(Row) + 15) & ~(size_t)15));
+    uint16_t *cnt = parent + (((size_t)V * 2 + 15) & ~(size_t)15) / 2;
+    __shared__ int s_nslow;
+    int *s_list = reinterpret_cast<int *>(cnt + (((size_t)V * 2 + 15) & ~(size_t)15) / 2);   // [slots] slow pairs
+    int *s_target = s_list + slots, *s_count = s_target + slots;                          // [slots] each
+    int *s_res = s_count + slots;                                                         // [slots][4]
+    if (tid == 0) s_nslow = 0;
+    __syncthreads();
+
+    const PairItem p = pair_item(a, bid * slots + slot);
+    const bool acu = b.cluster_mode == PTHR_CLUSTER_ACU;
+    const int cap = a.iter_cap > 0 ? a.iter_cap : 4 * V + 64;
+    const bool mine = p.live && yl < L;              // this lane holds rows
+    const int y = yl < L ? yl : L - 1;
+    const int yp = (y + 1) % L, ym = (y + L - 1) % L;
+    const int lp = sub * LN + yp, lm = sub * LN + ym;   // lanes of the y neighbours
+    uint32_t *A = b.spins + ((size_t)p.s * b.NLAT + p.la) * b.lat_words;
+    uint32_t *B = b.spins + ((size_t)p.s * b.NLAT + p.lb) * b.lat_words;
+
+    // ---- rows of q and of clone a's signs
+    uint32_t u[L];                                   // unlabelled sites
+    if (b.bits) {
+#pragma unroll
+        for (int z = 0; z < L; ++z) {
+            const int r = y + L * z, p0 = (y + z) & 1;
+            const uint32_t av = mine ? row_of_bits<L>(A, r, p0) : 0u, bv = mine ? row_of_bits<L>(B, r, p0) : 0u;
+            u[z] = av ^ bv;
+            if (yl < L) as[r] = (Row)av;
+        }
+    } else {
+        constexpr int ZB = rows_in_flight(L);
+#pragma unroll
+        for (int z0 = 0; z0 < L; z0 += ZB) {
+            uint32_t wa[ZB][2][W], wb[ZB][2][W];
+#pragma unroll
+            for (int i = 0; i < ZB; ++i)
+#pragma unroll
+                for (int c = 0; c < 2; ++c) {
+                    load_words<W>(A + (c * ROWS + y + L * (z0 + i)) * W, wa[i][c]);
+                    load_words<W>(B + (c * ROWS + y + L * (z0 + i)) * W, wb[i][c]);
+                }
+#pragma unroll
+            for (int i = 0; i < ZB; ++i) {
+                const int r = y + L * (z0 + i), p0 = (y + z0 + i) & 1;
+                const uint32_t av = row_of_words<L>(wa[i], p0), bv = row_of_words<L>(wb[i], p0);
+                u[z0 + i] = mine ? av ^ bv : 0u;
+                if (yl < L) as[r] = (Row)av;
+            }
+        }
+    }
+#pragma unroll
+    for (int z = 0; z < L; ++z) {
+        const int r = y + L * z;
+        if (yl < L) {
+            qs[r] = (Row)u[z];
+            Fs[r] = 0;
+        }
+    }
+    // ---- single-cluster move: the floor(u*n)-th q = -1 site in site order
+    int target = -1;
+    if (!acu && !a.label_only) {
+        int n = 0;
+#pragma unroll
+        for (int z = 0; z < L; ++z) n += __popc(u[z]);
+        for (int o = LN / 2; o > 0; o >>= 1) n += __shfl_xor_sync(FULLW, n, o);
+        int want = -1;
+        if (n > 0) {
+            const uint32_t w = philox_word0(p.seed, 0u, p.pair_id, p.emcs, TAG_SINGLE);
+            want = (int)(((unsigned long long)(w >> 8) * (unsigned long long)n) >> 24);
+        }
+        int seen = 0;                                // sites of the planes below z
+#pragma unroll
+        for (int z = 0; z < L; ++z) {
+            const int c = __popc(u[z]);
+            int incl = c;
+            for (int o = 1; o < LN; o <<= 1) {
+                const int t = __shfl_up_sync(FULLW, incl, o, LN);
+                if (yl >= o) incl += t;
+            }
+            const int first = seen + incl - c;
+            if (want >= first && want < first + c) {
+                uint32_t v = u[z];
+                for (int m = want - first; m > 0; --m) v &= v - 1u;
+                target = L * (y + L * z) + __ffs(v) - 1;
+            }
+            seen += __shfl_sync(FULLW, incl, LN - 1, LN);
+        }
+        for (int o = LN / 2; o > 0; o >>= 1) target = max(target, __shfl_xor_sync(FULLW, target, o));
+    }
+    __syncwarp();
+    // ---- sites with no equal neighbour
+    int32_t *labels = nullptr;
+    if (a.label_only && p.live) labels = a.labels_out + ((size_t)(p.s * b.NPAIR + p.P) * b.NT + p.k) * V;
+    PairStats st{0, 0, 0};
+    {
+        int niso = 0;
+#pragma unroll
+        for (int z = 0; z < L; ++z) {
+            const uint32_t q = u[z];
+            const uint32_t ex = ~(q ^ rot_next<L>(q)) & M;             // x and x + 1 equal
+            const uint32_t ey = ~(q ^ qs[yp + L * z]) | ~(q ^ qs[ym + L * z]);
+            const uint32_t ez = ~(q ^ u[(z + 1) % L]) | ~(q ^ u[(z + L - 1) % L]);
+            const uint32_t eq = ex | (ex << 1) | (ex >> (L - 1)) | ey | ez;
+            const uint32_t iso = M & ~eq;
+            if (mine) Fs[y + L * z] = (Row)iso;          // for now
+            niso += mine ? __popc(iso) : 0;
+        }
+#pragma unroll
+        for (int z = 0; z < L; ++z) u[z] = mine ? M & ~(uint32_t)Fs[y + L * z] : 0u;
+        // one site per lane and turn, so that the lanes draw their signs
+        // together (turns = the most such sites of one lane)
+        int z = -1;
+        uint32_t v = 0, f = 0;
+        while (mine) {
+            while (v == 0u && z < L) {
+                if (z >= 0) Fs[y + L * z] = (Row)f;
+                f = 0u;
+                if (++z < L) v = Fs[y + L * z];
+            }
+            if (z >= L) break;
+            const int x = 31 - __clz(v), i = L * (y + L * z) + x;
+            v ^= 1u << x;
+            if (a.label_only) labels[i] = i;
+            else if (acu ? cluster_sign(p, i) : i == target) f |= 1u << x;
+        }
+        __syncwarp();
+        for (int o = LN / 2; o > 0; o >>= 1) niso += __shfl_xor_sync(FULLW, niso, o);
+        st = PairStats{niso, niso > 0 ? 1 : 0, niso > 1 ? 1 : 0};
+    }
+    // ---- the other clusters, by their smallest site: in each turn the first
+    // unlabelled q = +1 site's cluster and the first q = -1 site's
+    using Fw = FloodWords<L>;
+    bool ok = true, slow = false;
+    int big0 = 0, big1 = 0;                              // largest cluster of each sign so far
+    bool flip0 = false, flip1 = false;                   // and whether it flips
+    if (Fw::PACKED) {
+#pragma unroll
+        for (int z = 0; z < L; ++z) {
+            const uint32_t q = qs[y + L * z];
+            u[z] = (u[z] & ~q) | ((u[z] & q) << 16);
+        }
+    }
+    uint32_t ur[L];
+#pragma unroll
+    for (int z = 0; z < L; ++z) ur[z] = __brev(u[z]);
+    for (int nf = 0; nf <= MAX_FLOODS; ++nf) {
+        // first sites; 0xFFFF: none (V < 2^16)
+        uint32_t key = 0xFFFFFFFFu;
+        {
+            int z0 = -1, z1 = -1;
+            uint32_t w0 = 0, w1 = 0;
+#pragma unroll
+            for (int z = L - 1; z >= 0; --z) {
+                if (Fw::PACKED) {
+                    if (u[z] & 0xFFFFu) { z0 = z; w0 = u[z]; }
+                    if (u[z] > 0xFFFFu) { z1 = z; w1 = u[z]; }
+                } else if (u[z]) {
+                    z0 = z;
+                    w0 = u[z];
+                }
+            }
+            if (z0 >= 0) key = (uint32_t)(L * (y + L * z0) + __ffs(w0) - 1);
+            if (Fw::PACKED) {
+                key &= 0xFFFFu;
+                key |= z1 >= 0 ? (uint32_t)(L * (y + L * z1) + __ffs(w1 >> 16) - 1) << 16 : 0xFFFF0000u;
+            }
+        }
+        for (int o = LN / 2; o > 0; o >>= 1) {
+            const uint32_t other = __shfl_xor_sync(FULLW, key, o);
+            key = Fw::PACKED ? __vminu2(key, other) : min(key, other);
+        }
+        const bool act = key != 0xFFFFFFFFu;
+        if (!__any_sync(FULLW, act)) break;
+        if (nf == MAX_FLOODS) { slow = act; break; }
+        const int lab[2] = {(int)(Fw::PACKED ? key & 0xFFFFu : key), (int)(Fw::PACKED ? key >> 16 : 0xFFFFu)};
+        uint32_t m[L], f[L];
+        int sign1 = 0;                                   // unpacked: the cluster's sign is -1
+        if (Fw::PACKED) {
+            // (a label 0xFFFF lies in no plane: V <= 16^3)
+            const int r0 = lab[0] / L, r1 = lab[1] / L, z0 = r0 / L, z1 = r1 / L;
+            const uint32_t b0 = yl == r0 - L * z0 ? 1u << (lab[0] - L * r0) : 0u;
+            const uint32_t b1 = yl == r1 - L * z1 ? 0x10000u << (lab[1] - L * r1) : 0u;
+#pragma unroll
+            for (int z = 0; z < L; ++z) {
+                m[z] = u[z];
+                f[z] = (z == z0 ? b0 : 0u) | (z == z1 ? b1 : 0u);
+            }
+        } else {
+            // one cluster at a time, of the sign of its first site
+            const int rs = act ? lab[0] / L : 0, xs = act ? lab[0] - rs * L : 0;
+            sign1 = (int)((qs[rs] >> xs) & 1u);
+            const uint32_t inv = sign1 ? 0u : FULLW;
+#pragma unroll
+            for (int z = 0; z < L; ++z) {
+                const int r = y + L * z;
+                m[z] = act ? u[z] & (qs[r] ^ inv) : 0u;
+                ur[z] = __brev(m[z]);
+                f[z] = act && yl < L && r == rs ? 1u << xs : 0u;
+            }
+        }
+        // passes over the rows, upwards and downwards in turn, until one
+        // changes nothing; four chains of L/4 rows advance side by side, since
+        // one row's shuffles, reversals and carries are a serial chain of about
+        // 90 cycles (on thermalised pairs four chains need 5% more row visits
+        // than one, and a quarter of the serial steps)
+        constexpr int CH = (L + 3) / 4;
+        bool more = true;
+        for (int it = 0; more && it < 2 * cap; ++it) {
+            uint32_t ch = 0;
+            if ((it & 1) == 0) {
+#pragma unroll
+                for (int v = 0; v < CH; ++v)
+#pragma unroll
+                    for (int z = v; z < L; z += CH) ch |= flood_row<L>(f, m, ur, z, lp, lm);
+            } else {
+#pragma unroll
+                for (int v = CH - 1; v >= 0; --v)
+#pragma unroll
+                    for (int z = v; z < L; z += CH) ch |= flood_row<L>(f, m, ur, z, lp, lm);
+            }
+            more = __any_sync(FULLW, ch != 0u);
+        }
+        if (more && act) ok = false;
+        int size = 0;                                    // both clusters' sites, 16 bits each
+#pragma unroll
+        for (int z = 0; z < L; ++z)
+            size += Fw::PACKED ? __popc(f[z] & 0xFFFFu) + (__popc(f[z] >> 16) << 16) : __popc(f[z]);
+        for (int o = LN / 2; o > 0; o >>= 1) size += __shfl_xor_sync(FULLW, size, o);
+        bool flip[2] = {false, false};                   // of the two clusters
+        bool holds[2] = {false, false};                  // the single move's target site
+        if (!acu) {
+#pragma unroll
+            for (int z = 0; z < L; ++z) {
+                const int x = target - L * (y + L * z);
+                if (yl < L && x >= 0 && x < L) {
+                    holds[0] = (f[z] >> x) & 1u;
+                    holds[1] = Fw::PACKED && ((f[z] >> (16 + x)) & 1u);
+                }
+            }
+        }
+        // even lanes draw the sign of one cluster, odd lanes of the other
+        const unsigned drawn = __ballot_sync(FULLW, acu && cluster_sign(p, lab[Fw::PACKED ? yl & 1 : 0]));
+#pragma unroll
+        for (int h = 0; h < (Fw::PACKED ? 2 : 1); ++h) {
+            const int sz = Fw::PACKED ? (h ? (int)((uint32_t)size >> 16) : size & 0xFFFF) : size;
+            if (sz > 0) add_size(st, sz);
+            if (acu) {
+                flip[h] = sz > 0 && ((drawn >> (sub * LN + h)) & 1u);
+            } else {
+                const unsigned any = __ballot_sync(FULLW, holds[h]);
+                flip[h] = ((any >> (sub * LN)) & (unsigned)((1ull << LN) - 1ull)) != 0u;
+            }
+            const int sign = Fw::PACKED ? h : sign1;
+            if (sz > (sign ? big1 : big0)) {
+                if (sign) { big1 = sz; flip1 = flip[h]; } else { big0 = sz; flip0 = flip[h]; }
+            }
+        }
+        if (a.label_only) {
+            if (mine) {
+#pragma unroll
+                for (int z = 0; z < L; ++z) as[y + L * z] = (Row)(f[z] & Fw::M);
+                if (Fw::PACKED) {
+#pragma unroll
+                    for (int z = 0; z < L; ++z) Fs[y + L * z] = (Row)(f[z] >> 16);
+                }
+                for (int z = 0; z < L; ++z) {
+#pragma unroll
+                    for (int h = 0; h < (Fw::PACKED ? 2 : 1); ++h) {
+                        uint32_t v = h ? Fs[y + L * z] : as[y + L * z];
+                        while (v) {
+                            const int x = 31 - __clz(v);
+                            v ^= 1u << x;
+                            labels[L * (y + L * z) + x] = lab[h];
+                        }
+                    }
+                }
+            }
+        } else if (flip[0] || flip[1]) {
+            const uint32_t k0 = flip[0] ? Fw::M : 0u, k1 = flip[1] ? Fw::M : 0u;
+#pragma unroll
+            for (int z = 0; z < L; ++z) {
+                const uint32_t v = Fw::PACKED ? (f[z] & k0) | ((f[z] >> 16) & k1) : f[z];
+                if (v) Fs[y + L * z] |= (Row)v;
+            }
+        }
+#pragma unroll
+        for (int z = 0; z < L; ++z) {
+            u[z] &= ~f[z];
+            if (Fw::PACKED) ur[z] = __brev(u[z]);
+        }
+    }
+    // ---- flips, energies and statistics; then, if the block has any, the pairs
+    // of many clusters (the whole block, one pair after another) and theirs
+#pragma unroll 1
+    for (int turn = 0; turn < 2; ++turn) {
+        if (turn == 1) {
+            if (slow && yl == 0) {
+                const int i = atomicAdd(&s_nslow, 1);
+                s_list[i] = slot;
+                s_target[i] = target;
+            }
+            __syncthreads();
+            const int nslow = s_nslow;
+            if (nslow == 0) return;
+            for (int i = 0; i < nslow; ++i) {
+                const int sl = s_list[i];
+                const PairItem ps = pair_item(a, bid * slots + sl);
+                PairStats r{0, 0, 0};
+                const bool good = union_find_pair<L, Row>(a, ps, s_target[i], rows + (size_t)sl * 3 * ROWS,
+                                                          rows + (size_t)sl * 3 * ROWS + 2 * ROWS, parent, cnt,
+                                                          cap, r);
+                if (tid == 0) {
+                    s_res[4 * sl] = good;
+                    s_res[4 * sl + 1] = r.nclus;
+                    s_res[4 * sl + 2] = r.top1;
+                    s_res[4 * sl + 3] = r.top2;
+                }
+                __syncthreads();
+            }
+            if (slow) {
+                ok = s_res[4 * slot] != 0;
+                st = PairStats{s_res[4 * slot + 1], s_res[4 * slot + 2], s_res[4 * slot + 3]};
+            }
+        }
+        if (__any_sync(FULLW, slow) == (turn == 1))
+            finish_pair<L, Row>(a, p, qs, as, Fs, list, s_count + slot, sub, yl, ok, !slow && flip0 != flip1, st);
+    }
 }
 
-// parent, cnt [V] int; both clones [LW]; root flags [V] bytes; q and clone-a
-// rows [L*L]; the row-count scan of the single-cluster move [<= 1024] int
 template <int L>
-size_t cluster_smem(void) {
-    using Gm = Geom<L>;
-    return (size_t)8 * Gm::V + (size_t)8 * Gm::LAT_WORDS + (size_t)((Gm::V + 3) & ~3) +
-           (size_t)8 * L * L + (size_t)4 * 1024 + 16;
+__global__ void __launch_bounds__(CLUSTER_MAX_THREADS, L <= 8 || L > 16 ? 4 : 5) cluster_kernel(ClusterArgs a) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    cluster_block<L>(a, blockIdx.x, smem);
 }
 
 template <int L>
 cudaError_t launch_cluster_L(const ClusterArgs &a, int threads, cudaStream_t st) {
     static bool configured = false;
     if (!configured) {
-        cudaError_t e = allow_max_dynamic_smem(cluster_kernel<L, false>);
-        if (e == cudaSuccess) e = allow_max_dynamic_smem(cluster_kernel<L, true>);
+        cudaError_t e = allow_max_dynamic_smem(cluster_kernel<L>);
         if (e != cudaSuccess) return e;
         configured = true;
     }
-    const int blocks = a.sample_count * a.b.NPAIR * a.b.n_acu;
+    const int blocks = cluster_blocks_for(L, a.sample_count * a.b.NPAIR * a.b.n_acu, threads);
     if (blocks <= 0) return cudaSuccess;
-    if (a.iter_cap > 0)
-        cluster_kernel<L, true><<<blocks, threads, cluster_smem<L>(), st>>>(a);
-    else
-        cluster_kernel<L, false><<<blocks, threads, cluster_smem<L>(), st>>>(a);
+    cluster_kernel<L><<<blocks, threads, cluster_smem<L>(threads), st>>>(a);
     return cudaGetLastError();
 }
 
 // The cluster step of a mixed-L group (see kernels.cuh): the blocks of every
-// batch's cluster launch, dispatching on its lattice size; block size = the
-// largest of the group (every loop strides by the block size).
-__global__ void __launch_bounds__(512, 2) group_cluster_kernel(GroupClusterArgs g) {
+// batch's cluster launch, dispatching on its lattice size; one block size for
+// the group.
+__global__ void __launch_bounds__(CLUSTER_MAX_THREADS, 5) group_cluster_kernel(GroupClusterArgs g) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ ClusterArgs ca;
     const int i = group_member(g.off, g.n, (int)blockIdx.x);
@@ -508,13 +906,19 @@ __global__ void __launch_bounds__(512, 2) group_cluster_kernel(GroupClusterArgs 
     __syncthreads();
     const int bid = (int)blockIdx.x - g.off[i];
     switch (ca.b.L) {
-#define X(LL) case LL: cluster_block<LL, false>(ca, bid, smem); break;
+#define X(LL) case LL: cluster_block<LL>(ca, bid, smem); break;
         X(4) X(6) X(8) X(10) X(12) X(14) X(16)
 #undef X
     }
 }
 
 }  // namespace
+
+int cluster_blocks_for(int L, int pairs, int threads) {
+    const int lanes = L <= 4 ? 4 : (L <= 8 ? 8 : (L <= 16 ? 16 : 32));
+    const int slots = (threads / 32) * (32 / lanes);
+    return (pairs + slots - 1) / slots;
+}
 
 cudaError_t launch_group_cluster(const GroupClusterArgs &g, int blocks, int threads, size_t smem, cudaStream_t st) {
     if (blocks <= 0) return cudaSuccess;
@@ -528,8 +932,8 @@ cudaError_t launch_group_cluster(const GroupClusterArgs &g, int blocks, int thre
     return cudaGetLastError();
 }
 
-size_t cluster_smem_bytes_for(int L) {
-#define X(LL) if (L == LL) return cluster_smem<LL>();
+size_t cluster_smem_bytes_for(int L, int threads) {
+#define X(LL) if (L == LL) return cluster_smem<LL>(threads);
     PTHR_FOR_EACH_L(X)
 #undef X
     return 0;

@@ -31,10 +31,12 @@ struct ClusterArgs {
     int sample_first, sample_count;
     int label_only;          // 1: only write labels (no flip, no energies)
     int32_t *labels_out;     // optional [S][NPAIR][NT][V] canonical labels
-    int iter_cap;            // bound on every union-find loop (> 0)
+    int iter_cap;            // > 0: bound on every labelling loop (0: 4V + 64)
 };
+constexpr int CLUSTER_MAX_THREADS = 128;   // per block: its warps work on pairs of their own
 cudaError_t launch_cluster(const ClusterArgs &a, int threads, cudaStream_t st);
-size_t cluster_smem_bytes_for(int L);
+size_t cluster_smem_bytes_for(int L, int threads);
+int cluster_blocks_for(int L, int pairs, int threads);   // blocks for that many pairs
 
 // exchange.cu
 cudaError_t launch_swap(const Batch &b, int flags, int first, int count, cudaStream_t st);
