@@ -93,26 +93,21 @@ __device__ __forceinline__ uint32_t row_of_bits(const uint32_t *S, int r, int p0
 // Row r = y + L z of the bit mask where lattices A and B differ (q_i = -1):
 // bit x set iff the spins at x + L r differ.  A and B in the storage layout
 // (BITS: the bit layout, else the byte layout).
-template <int L, bool BITS = false>
+template <int L, bool BITS>
 __device__ __forceinline__ uint32_t diff_row(const uint32_t *A, const uint32_t *B, int r) {
     using Gm = Geom<L>;
-    constexpr int W = Gm::W, ROWS = Gm::ROWS, Lh = Gm::Lh;
-    uint32_t bits[2];
+    constexpr int W = Gm::W, ROWS = Gm::ROWS;
+    const int p0 = ((r % L) + (r / L)) & 1;     // x parity of colour 0 in this row
+    if (BITS) return row_of_bits<L>(A, r, p0) ^ row_of_bits<L>(B, r, p0);
+    uint32_t w[2][W], v[W];
 #pragma unroll
     for (int c = 0; c < 2; ++c) {
-        uint32_t acc = 0;
+        load_words<W>(A + (c * ROWS + r) * W, w[c]);
+        load_words<W>(B + (c * ROWS + r) * W, v);
 #pragma unroll
-        for (int j = 0; j < W; ++j) {
-            const int w = (c * ROWS + r) * W + j;
-            if (BITS)
-                acc |= (((A[w >> 3] ^ B[w >> 3]) >> (4 * (w & 7))) & 0xFu) << (4 * j);
-            else
-                acc |= sign_nibble(A[w] ^ B[w]) << (4 * j);
-        }
-        bits[c] = acc & ((1u << Lh) - 1u);
+        for (int j = 0; j < W; ++j) w[c][j] ^= v[j];
     }
-    const int p0 = ((r % L) + (r / L)) & 1;     // x parity of colour 0 in this row
-    return (spread_bits(bits[0]) << p0) | (spread_bits(bits[1]) << (p0 ^ 1));
+    return row_of_words<L>(w, p0);
 }
 
 }  // namespace pthr

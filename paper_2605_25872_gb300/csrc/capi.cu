@@ -869,7 +869,7 @@ pthr_status group_fused_emcs(pthr_batch *const *batches, int n, cudaStream_t st,
         gm.off[gm.n] = m_blocks;
         ++gm.n;
         m_blocks += (c->n_samples * c->n_temps + 7) / 8;
-        if (measure_smem_bytes_for(c->L) > m_smem) m_smem = measure_smem_bytes_for(c->L);
+        if (measure_smem_bytes_for(c->L, c->n_replicas) > m_smem) m_smem = measure_smem_bytes_for(c->L, c->n_replicas);
     }
     gs.off[gs.n] = sw_blocks;
     gc.off[gc.n] = cl_blocks;

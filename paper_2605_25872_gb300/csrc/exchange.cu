@@ -99,110 +99,147 @@ constexpr int MEASURE_WARPS = 8;   // (sample, temperature) items per measuremen
 // read once, row by row, so a warp's loads are consecutive words) into its
 // shared-memory slot, then counts the sites with q_i = -1 and the forward
 // links (i, i + mu) with q_i != q_{i+mu} by popcounts of each row against
-// its rotation (x), its y + 1 row and its z + 1 row.  Lane P keeps pair P's
-// counts.  Then the FP64 quantities of the groups and pairs are evaluated on
-// separate lanes, and lane 0 adds them to the accumulators in the fixed
-// order (groups, then pairs) with one IEEE rounding per operation.
+// its rotation (x), its y + 1 row and its z + 1 row.
+//
+// The FP64 part is done for the block's eight items together: this GPU issues
+// 1.7 FP64 lanes per SM and clock, so an FP64 instruction costs a warp 19
+// cycles however few of its lanes work, and the divisions and sums of one item
+// (about 80 instructions) on a warp of its own would take longer than its rows.
+// First one thread per (item, group) and (item, pair) forms the terms, then one
+// thread per (item, accumulator) adds them in the fixed order (groups, then
+// pairs) with one IEEE rounding per operation.  Measured, one launch, against
+// the FP64 part on every item's own warp: L = 12, 1024 x 24 items 60 us
+// (101 us); L = 8, 256 x 16 9.6 us (21.8 us); L = 16, 512 x 32 63 us (80 us);
+// the spins alone take 33 us (226 MB) at L = 12 and 40 us (268 MB) at L = 16.
+__host__ __device__ inline size_t measure_smem_words(int L, int NR) {
+    const int NP = NR / 2 > 0 ? NR / 2 : 1;
+    return (size_t)MEASURE_WARPS * (L * L + 4 * NP) + (size_t)MEASURE_WARPS * (2 * NR + 6 * NP) * 2;
+}
+
 template <int L>
 __device__ __forceinline__ void measure_block(const Batch &b, int first, int count, int chaos, int bid,
                                               unsigned char *smem) {
     using Gm = Geom<L>;
     constexpr int V = Gm::V, ROWS = Gm::ROWS;
-    uint32_t *s_q = reinterpret_cast<uint32_t *>(smem);   // [MEASURE_WARPS][ROWS]
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const int item = bid * MEASURE_WARPS + wid;
-    if (item >= count * b.NT) return;                 // warp-uniform
-    const int s = first + item / b.NT, k = item % b.NT;
-    if (!PTHR_DCHECK(b.status, s >= 0 && s < b.S)) return;
-    if (!b.active[s]) return;
-    const int32_t *perm = b.perm + (size_t)s * b.NR * b.NSLOT;
-    const int lw = b.lat_words;                       // storage words per lattice
-    const uint32_t *spins = b.spins + (size_t)s * b.NLAT * lw;
-    uint32_t *qr = s_q + wid * ROWS;
-    int tn = 0, td = 0, tc = 0;                       // pair `lane`'s counts
-    for (int P = 0; P < b.NPAIR; ++P) {
-        const int la = 2 * P * b.NSLOT + perm[2 * P * b.NSLOT + k];
-        const int lb = (2 * P + 1) * b.NSLOT + perm[(2 * P + 1) * b.NSLOT + k];
-        if (!PTHR_DCHECK(b.status, la >= 2 * P * b.NSLOT && la < (2 * P + 1) * b.NSLOT &&
-                                    lb >= (2 * P + 1) * b.NSLOT && lb < (2 * P + 2) * b.NSLOT)) return;
-        const uint32_t *A = spins + (size_t)la * lw, *B = spins + (size_t)lb * lw;
-        int nneg = 0, ndiff = 0, cneg = 0;
-        for (int r = lane; r < ROWS; r += 32) {
-            const uint32_t q = b.bits ? diff_row<L, true>(A, B, r) : diff_row<L>(A, B, r);
-            qr[r] = q;
-            nneg += __popc(q);
+    const int NR = b.NR, NP = b.NPAIR, NPs = NP > 0 ? NP : 1;
+    // terms of the accumulators [item][2 NR + 6 NP], counts [item][pair][4], rows [item][ROWS]
+    double *s_v = reinterpret_cast<double *>(smem);
+    int *s_c = reinterpret_cast<int *>(s_v + MEASURE_WARPS * (2 * NR + 6 * NPs));
+    uint32_t *s_q = reinterpret_cast<uint32_t *>(s_c + MEASURE_WARPS * 4 * NPs);
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const int items = count * b.NT;
+    // ---- counts of this warp's item
+    {
+        const int item = bid * MEASURE_WARPS + wid;
+        const int s = first + item / b.NT, k = item % b.NT;
+        if (item < items && PTHR_DCHECK(b.status, s >= 0 && s < b.S) && b.active[s]) {   // warp-uniform
+            const int32_t *perm = b.perm + (size_t)s * NR * b.NSLOT;
+            const int lw = b.lat_words;                       // storage words per lattice
+            const uint32_t *spins = b.spins + (size_t)s * b.NLAT * lw;
+            uint32_t *qr = s_q + wid * ROWS;
+            for (int P = 0; P < NP; ++P) {
+                int la = 2 * P * b.NSLOT + perm[2 * P * b.NSLOT + k];
+                int lb = (2 * P + 1) * b.NSLOT + perm[(2 * P + 1) * b.NSLOT + k];
+                if (!PTHR_DCHECK(b.status, la >= 2 * P * b.NSLOT && la < (2 * P + 1) * b.NSLOT &&
+                                            lb >= (2 * P + 1) * b.NSLOT && lb < (2 * P + 2) * b.NSLOT)) la = lb = 0;
+                const uint32_t *A = spins + (size_t)la * lw, *B = spins + (size_t)lb * lw;
+                int nneg = 0, ndiff = 0, cneg = 0;
+                if (b.bits) {
+                    for (int r = lane; r < ROWS; r += 32) {
+                        const uint32_t q = diff_row<L, true>(A, B, r);
+                        qr[r] = q;
+                        nneg += __popc(q);
+                    }
+                } else {
+#pragma unroll 4
+                    for (int r = lane; r < ROWS; r += 32) {   // four rows' loads in flight
+                        const uint32_t q = diff_row<L, false>(A, B, r);
+                        qr[r] = q;
+                        nneg += __popc(q);
+                    }
+                }
+                __syncwarp();
+                for (int r = lane; r < ROWS; r += 32) {
+                    const int y = r % L, z = r / L;
+                    const uint32_t q = qr[r];
+                    const uint32_t qy = qr[((y + 1) % L) + L * z], qz = qr[y + L * ((z + 1) % L)];
+                    ndiff += __popc(q ^ rot_next<L>(q)) + __popc(q ^ qy) + __popc(q ^ qz);
+                }
+                if (chaos) {
+                    // temperature chaos: clone of group 2P at T_0 against group 2P+1 at T_k
+                    const uint32_t *A0 = spins + (size_t)(2 * P * b.NSLOT + perm[2 * P * b.NSLOT]) * lw;
+                    for (int r = lane; r < ROWS; r += 32)
+                        cneg += __popc(b.bits ? diff_row<L, true>(A0, B, r) : diff_row<L, false>(A0, B, r));
+                }
+                __syncwarp();                                 // qr is reused by the next pair
+                nneg = __reduce_add_sync(0xffffffffu, nneg);
+                ndiff = __reduce_add_sync(0xffffffffu, ndiff);
+                cneg = __reduce_add_sync(0xffffffffu, cneg);
+                if (lane == 0) {
+                    int *c = s_c + 4 * (wid * NPs + P);
+                    c[0] = nneg;
+                    c[1] = ndiff;
+                    c[2] = cneg;
+                }
+            }
         }
-        __syncwarp();
-        for (int r = lane; r < ROWS; r += 32) {
-            const int y = r % L, z = r / L;
-            const uint32_t q = qr[r];
-            const uint32_t qy = qr[((y + 1) % L) + L * z], qz = qr[y + L * ((z + 1) % L)];
-            ndiff += __popc(q ^ rot_next<L>(q)) + __popc(q ^ qy) + __popc(q ^ qz);
-        }
-        if (chaos) {
-            // temperature chaos: clone of group 2P at T_0 against group 2P+1 at T_k
-            const uint32_t *A0 = spins + (size_t)(2 * P * b.NSLOT + perm[2 * P * b.NSLOT]) * lw;
-            for (int r = lane; r < ROWS; r += 32)
-                cneg += __popc(b.bits ? diff_row<L, true>(A0, B, r) : diff_row<L>(A0, B, r));
-        }
-        __syncwarp();                                 // qr is reused by the next pair
-        nneg = __reduce_add_sync(0xffffffffu, nneg);
-        ndiff = __reduce_add_sync(0xffffffffu, ndiff);
-        cneg = __reduce_add_sync(0xffffffffu, cneg);
-        if (lane == P) { tn = nneg; td = ndiff; tc = cneg; }
     }
-    // per-group energy density on lane g, per-pair overlaps on lane P
-    double e = 0.0, q = 0.0, ql = 0.0, S = 0.0, qc = 0.0;
-    // e = H / V (exact scaling when V is a power of two); q, q_l and T_k
-    // come from the creation-time tables of the same divisions
-    if (lane < b.NR) {
-        const int lat = lane * b.NSLOT + perm[lane * b.NSLOT + k];
+    __syncthreads();
+    // ---- terms: e and e^2 of every (item, group); q, q^2, q_l, S, q^4 and the
+    // chaos q^2 of every (item, pair).  e = H / V is an exact scaling when V is
+    // a power of two; q, q_l and T_k come from the creation-time tables of the
+    // same divisions.
+    const int NV = 2 * NR + 6 * NPs;                          // terms per item
+    for (int i = tid; i < MEASURE_WARPS * NR; i += blockDim.x) {
+        const int w = i / NR, g = i - w * NR, item = bid * MEASURE_WARPS + w;
+        if (item >= items) break;
+        const int s = first + item / b.NT, k = item % b.NT;
+        if (!b.active[s]) continue;
+        const int lat = g * b.NSLOT + b.perm[((size_t)s * NR + g) * b.NSLOT + k];
         const double H = b.E[(size_t)s * b.NLAT + lat];
-        e = ((V & (V - 1)) == 0) ? __dmul_rn(H, 1.0 / (double)V) : __ddiv_rn(H, (double)V);
+        const double e = ((V & (V - 1)) == 0) ? __dmul_rn(H, 1.0 / (double)V) : __ddiv_rn(H, (double)V);
+        s_v[w * NV + g] = e;
+        s_v[w * NV + NR + g] = __dmul_rn(e, e);
     }
-    if (lane < b.NPAIR) {
-        const double Tk = b.tabT[k];
-        const int la = 2 * lane * b.NSLOT + perm[2 * lane * b.NSLOT + k];
+    for (int i = tid; i < MEASURE_WARPS * NP; i += blockDim.x) {
+        const int w = i / NP, P = i - w * NP, item = bid * MEASURE_WARPS + w;
+        if (item >= items) break;
+        const int s = first + item / b.NT, k = item % b.NT;
+        if (!b.active[s]) continue;
+        const int *c = s_c + 4 * (w * NPs + P);
+        int tn = c[0], td = c[1], tc = c[2];
         if (!PTHR_DCHECK(b.status, tn >= 0 && tn <= V && td >= 0 && td <= 3 * V && tc >= 0 && tc <= V)) {
             tn = 0; td = 0; tc = 0;
         }
-        q = b.tabQ[tn];
-        ql = b.tabQl[td];
+        const double q = b.tabQ[tn], ql = b.tabQl[td], qc = b.tabQ[tc];
+        const int la = 2 * P * b.NSLOT + b.perm[((size_t)s * NR + 2 * P) * b.NSLOT + k];
         const double Ha = b.E[(size_t)s * b.NLAT + la];
-        S = __dadd_rn(__ddiv_rn(Ha, 3.0 * (double)V), __ddiv_rn(__dsub_rn(1.0, ql), Tk));
-        qc = b.tabQ[tc];
+        const double q2 = __dmul_rn(q, q);
+        double *v = s_v + w * NV + 2 * NR + P;
+        v[0] = q;
+        v[NPs] = q2;
+        v[2 * NPs] = ql;
+        v[3 * NPs] = __dadd_rn(__ddiv_rn(Ha, 3.0 * (double)V), __ddiv_rn(__dsub_rn(1.0, ql), b.tabT[k]));
+        v[4 * NPs] = __dmul_rn(__dmul_rn(q2, q), q);
+        if (chaos) v[5 * NPs] = __dmul_rn(qc, qc);
     }
-    double *o = b.obs + ((size_t)s * b.NT + k) * PTHR_NOBS;
-    double se = 0.0, se2 = 0.0;
-    if (lane == 0) { se = o[1]; se2 = o[2]; }
-    for (int g = 0; g < b.NR; ++g) {
-        const double eg = __shfl_sync(0xffffffffu, e, g);
-        if (lane == 0) {
-            se = __dadd_rn(se, eg);
-            se2 = __dadd_rn(se2, __dmul_rn(eg, eg));
-        }
-    }
-    if (lane == 0) {
-        o[0] = __dadd_rn(o[0], 1.0);
-        o[1] = se;
-        o[2] = se2;
-    }
-    double *c = b.chaos + ((size_t)s * b.NT + k) * 2;
-    for (int P = 0; P < b.NPAIR; ++P) {
-        const double qP = __shfl_sync(0xffffffffu, q, P), qlP = __shfl_sync(0xffffffffu, ql, P);
-        const double SP = __shfl_sync(0xffffffffu, S, P), qcP = __shfl_sync(0xffffffffu, qc, P);
-        if (lane == 0) {
-            const double q2 = __dmul_rn(qP, qP);
-            o[3] = __dadd_rn(o[3], qP);
-            o[4] = __dadd_rn(o[4], q2);
-            o[5] = __dadd_rn(o[5], qlP);
-            o[6] = __dadd_rn(o[6], SP);
-            o[7] = __dadd_rn(o[7], __dmul_rn(__dmul_rn(q2, qP), qP));
-            if (chaos) {
-                c[0] = __dadd_rn(c[0], 1.0);
-                c[1] = __dadd_rn(c[1], __dmul_rn(qcP, qcP));
-            }
-        }
+    __syncthreads();
+    // ---- sums: thread = (item, accumulator); accumulators 8 and 9: chaos
+    const int NA = chaos ? PTHR_NOBS + 2 : PTHR_NOBS;
+    for (int i = tid; i < MEASURE_WARPS * NA; i += blockDim.x) {
+        const int w = i / NA, acc = i - w * NA, item = bid * MEASURE_WARPS + w;
+        if (item >= items) break;
+        const int s = first + item / b.NT, k = item % b.NT;
+        if (!b.active[s]) continue;
+        const double *v = s_v + w * NV;
+        double *o = acc < PTHR_NOBS ? b.obs + ((size_t)s * b.NT + k) * PTHR_NOBS + acc
+                                    : b.chaos + ((size_t)s * b.NT + k) * 2 + (acc - PTHR_NOBS);
+        const bool ones = acc == 0 || acc == PTHR_NOBS;       // counters
+        const int n = acc == 0 ? 1 : (acc <= 2 ? NR : NP);
+        const double *t = acc <= 2 ? v + (acc == 2 ? NR : 0) : v + 2 * NR + (acc == PTHR_NOBS + 1 ? 5 : acc - 3) * NPs;
+        double sum = *o;
+        for (int j = 0; j < n; ++j) sum = __dadd_rn(sum, ones ? 1.0 : t[j]);
+        *o = sum;
     }
 }
 
@@ -270,7 +307,7 @@ cudaError_t launch_group_measure(const GroupBatchArgs &g, int blocks, size_t sme
     return cudaGetLastError();
 }
 
-size_t measure_smem_bytes_for(int L) { return (size_t)MEASURE_WARPS * L * L * 4; }
+size_t measure_smem_bytes_for(int L, int n_replicas) { return measure_smem_words(L, n_replicas) * 4; }
 
 cudaError_t launch_swap(const Batch &b, int flags, int first, int count, cudaStream_t st) {
     if (b.NR > 32 || b.NSLOT > MAX_SLOT) return cudaErrorInvalidValue;
@@ -291,7 +328,7 @@ cudaError_t launch_measure(const Batch &b, int first, int count, int chaos, cuda
     if (items <= 0) return cudaSuccess;
     const int blocks = (int)((items + MEASURE_WARPS - 1) / MEASURE_WARPS);
 #define X(LL) if (b.L == LL) { \
-        measure_kernel<LL><<<blocks, 32 * MEASURE_WARPS, measure_smem_bytes_for(LL), st>>>(b, first, count, chaos); \
+        measure_kernel<LL><<<blocks, 32 * MEASURE_WARPS, measure_smem_bytes_for(LL, b.NR), st>>>(b, first, count, chaos); \
         return cudaGetLastError(); }
     PTHR_FOR_EACH_L(X)
 #undef X

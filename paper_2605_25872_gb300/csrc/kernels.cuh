@@ -64,7 +64,7 @@ cudaError_t launch_group_sweep(const GroupSweepArgs &g, int rule, int blocks, in
 cudaError_t launch_group_cluster(const GroupClusterArgs &g, int blocks, int threads, size_t smem, cudaStream_t st);
 cudaError_t launch_group_swap(const GroupBatchArgs &g, int blocks, int threads, size_t smem, cudaStream_t st);
 cudaError_t launch_group_measure(const GroupBatchArgs &g, int blocks, size_t smem, cudaStream_t st);
-size_t measure_smem_bytes_for(int L);
+size_t measure_smem_bytes_for(int L, int n_replicas);
 
 // Block index of a group launch -> batch index (static indices only).
 __device__ __forceinline__ int group_member(const int (&off)[GROUP_MAX + 1], int n, int blk) {
