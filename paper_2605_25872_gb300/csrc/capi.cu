@@ -160,6 +160,8 @@ Layout make_layout(const pthr_config *c) {
     return l;
 }
 
+constexpr int GPU_SMS = 152;   // GB300
+
 // Kernel shapes.  Sweep: lattices per block K (PT / reservoir); Gt 4-site
 // groups per lattice lane (divides G, <= 512); P lattice lanes of KT
 // lattices each (KT one of the compiled variants); threads = P * Gt.
@@ -178,13 +180,32 @@ int default_k(const pthr_config *c, int total_entries) {
 
 // forced_kt > 0: lattices per thread fixed (the mixed-L group sweep compiles
 // one value per lattice size); the lattices per block then follow from it.
-SweepShape sweep_shape(const pthr_batch *b, int forced_kt = 0) {
+// samples, res: the launch's samples and whether its long blocks are the
+// reservoir's (240 sweeps per EMCS against 10).
+SweepShape sweep_shape(const pthr_batch *b, int forced_kt, int samples, bool res) {
     const pthr_config *c = &b->cfg;
     SweepShape sh{};
     const int npt = c->n_replicas * c->n_temps;
     const int nres = c->n_replicas * (c->n_res > 0 ? c->n_res : 1);
-    sh.K_pt = b->tuning.pt_lattices_per_block > 0 ? b->tuning.pt_lattices_per_block : default_k(c, npt);
-    sh.K_res = b->tuning.res_lattices_per_block > 0 ? b->tuning.res_lattices_per_block : default_k(c, nres);
+    sh.K_pt = default_k(c, npt);
+    sh.K_res = default_k(c, nres);
+    const int long_blocks = samples * (res ? (nres + sh.K_res - 1) / sh.K_res : (npt + sh.K_pt - 1) / sh.K_pt);
+    if (long_blocks < GPU_SMS && forced_kt == 0) {
+        // fewer long blocks than SMs: smaller blocks, and where a thread owns
+        // one group of a colour (L <= 16) few enough lattices per thread to
+        // keep its couplings in registers.  One EMCS alone / three batches on
+        // three streams: L = 14, 20 samples 0.81 / 0.62 ms (16 lattices per
+        // block: 3.05 / 1.02 ms); L = 18 MicSA, 24 samples 3.1 / 1.8 ms (5.5 /
+        // 1.9 ms; 4 lattices: 2.2 / 2.0 ms); L = 16, 64 samples' reservoir
+        // sweeps 1.62 ms (3.1 ms).  From one block per SM on the larger blocks
+        // stay: their couplings serve more updates.
+        const bool one_group = sweep_groups_for(c->L) <= 512;
+        const int most = one_group ? 4 : 8;
+        if (sh.K_res > most) sh.K_res = most;
+        if (one_group && sh.K_pt > most) sh.K_pt = most;
+    }
+    if (b->tuning.pt_lattices_per_block > 0) sh.K_pt = b->tuning.pt_lattices_per_block;
+    if (b->tuning.res_lattices_per_block > 0) sh.K_res = b->tuning.res_lattices_per_block;
     if (sh.K_pt > npt) sh.K_pt = npt;
     if (sh.K_res > nres) sh.K_res = nres;
     const int G = sweep_groups_for(c->L);
@@ -225,7 +246,7 @@ struct SweepLaunch { SweepArgs a; int blocks, threads, KT; size_t smem; };
 pthr_status sweep_launch(pthr_batch *b, int n_pt, int n_res, int first, int count, int pretherm,
                          int forced_kt, SweepLaunch *out) {
     const pthr_config *c = &b->cfg;
-    SweepShape sh = sweep_shape(b, forced_kt);
+    SweepShape sh = sweep_shape(b, forced_kt, count, c->n_res > 0 && n_res > 0);
     SweepArgs a{};
     a.b = b->dev;
     a.n_pt_sweeps = n_pt;
@@ -263,8 +284,6 @@ pthr_status do_sweep(pthr_batch *b, int n_pt, int n_res, int first, int count, i
         CUDA_TRY(b, launch_advance_pretherm(b->dev, first, count, n_res, b->stream), "pretherm counter");
     return PTHR_OK;
 }
-
-constexpr int GPU_SMS = 152;   // GB300
 
 // Threads per cluster-move block: whole warps, each with one to eight pairs
 // (larger requests run as blocks of CLUSTER_MAX_THREADS).  By default the
@@ -492,7 +511,7 @@ PTHR_API pthr_status pthr_set_tuning(pthr_batch *b, const pthr_tuning *t) {
         return fail(b, PTHR_E_INVAL, "tuning out of range");
     pthr_tuning old = b->tuning;
     b->tuning = nt;
-    SweepShape sh = sweep_shape(b);
+    SweepShape sh = sweep_shape(b, 0, b->cfg.n_samples, b->cfg.er_on != 0);
     const size_t smem = sweep_smem_bytes_for(b->cfg.L, sh.K_pt > sh.K_res ? sh.K_pt : sh.K_res);
     if (smem > 220 * 1024) {
         b->tuning = old;
@@ -521,7 +540,7 @@ PTHR_API pthr_status pthr_set_update_rule(pthr_batch *b, int rule) {
 
 PTHR_API pthr_status pthr_get_tuning(const pthr_batch *b, pthr_tuning *t) {
     if (!b || !t) return fail(nullptr, PTHR_E_INVAL, "NULL argument");
-    SweepShape sh = sweep_shape(b);
+    SweepShape sh = sweep_shape(b, 0, b->cfg.n_samples, b->cfg.er_on != 0);
     t->pt_lattices_per_block = sh.K_pt;
     t->res_lattices_per_block = sh.K_res;
     t->sweep_threads = sh.threads;

@@ -30,7 +30,7 @@ __global__ void __launch_bounds__(512, 1) group_sweep_kernel(GroupSweepArgs g) {
     __syncthreads();
     const int bid = (int)blockIdx.x - g.off[i];
     switch (sa.b.L) {
-#define X(LL) case LL: sweep_detail::sweep_block<LL, RULE, group_kt_of(LL)>(sa, bid, smem); break;
+#define X(LL) case LL: sweep_detail::sweep_block<LL, RULE, group_kt_of(LL), false>(sa, bid, smem); break;
         PTHR_GROUP_L(X)
 #undef X
     }

@@ -30,6 +30,7 @@ namespace pthr {
 namespace sweep_detail {
 
 constexpr int MAXK = 64;   // lattices per block
+constexpr int HOIST_KT = 4;   // lattices per thread up to which the couplings stay in registers
 
 // 32x32 -> 64-bit product as one wide multiply.
 __device__ __forceinline__ void mul_wide(uint32_t a, uint32_t b, uint32_t &hi, uint32_t &lo) {
@@ -203,6 +204,166 @@ __device__ __forceinline__ void group_fields(const uint32_t *S, const GroupGeo &
     }
 }
 
+// Couplings of the four sites of group g, colour c, as packed pairs (sites 0,1
+// and 2,3): +x, -x (or aligned, shifted x), +y, -y, +z, -z.
+template <int L, int RULE>
+__device__ __forceinline__ void sweep_couplings(const float *Js, const GroupGeo &q, int g, int c, f2 (&Jp)[2][6]) {
+    using Gm = Geom<L>;
+    constexpr int W = Gm::W, ROWS = Gm::ROWS, Lh = Gm::Lh, LB = Gm::LAT_BYTES;
+                    const int j = g % W;
+                    const int cc = c ^ 1;
+                    const int r = g / W;
+                    const int y = r % L, z = r / L;
+                    const int rym = ((y + L - 1) % L) + L * z, rzm = y + L * ((z + L - 1) % L);
+                    // couplings of the group's 4 sites: +x,-x,+y,-y,+z,-z
+                    float Jc[4][6];
+                    if (Gm::FULL) {
+                        // no row padding: the four sites' couplings of every
+                        // direction but -x are one aligned 16-byte load
+                        const float4 px = *reinterpret_cast<const float4 *>(Js + 4 * q.own);
+                        const float4 py = *reinterpret_cast<const float4 *>(Js + LB + 4 * q.own);
+                        const float4 pz = *reinterpret_cast<const float4 *>(Js + 2 * LB + 4 * q.own);
+                        const float4 my = *reinterpret_cast<const float4 *>(
+                            Js + LB + 4 * ((cc * ROWS + rym) * W) + 4 * j);
+                        const float4 mz = *reinterpret_cast<const float4 *>(
+                            Js + 2 * LB + 4 * ((cc * ROWS + rzm) * W) + 4 * j);
+                        const float vpx[4] = {px.x, px.y, px.z, px.w}, vpy[4] = {py.x, py.y, py.z, py.w};
+                        const float vpz[4] = {pz.x, pz.y, pz.z, pz.w}, vmy[4] = {my.x, my.y, my.z, my.w};
+                        const float vmz[4] = {mz.x, mz.y, mz.z, mz.w};
+    #pragma unroll
+                        for (int kk = 0; kk < 4; ++kk) {
+                            const int m = 4 * j + kk;
+                            const int mxm = q.par ? m : (m + Lh - 1) % Lh;
+                            Jc[kk][0] = vpx[kk];
+                            Jc[kk][1] = Js[4 * ((cc * ROWS + r) * W) + mxm];
+                            Jc[kk][2] = vpy[kk];
+                            Jc[kk][3] = vmy[kk];
+                            Jc[kk][4] = vpz[kk];
+                            Jc[kk][5] = vmz[kk];
+                        }
+                    } else {
+    #pragma unroll
+                        for (int kk = 0; kk < 4; ++kk) {
+                            int m = 4 * j + kk;
+                            if (m >= Lh) m = Lh - 1;
+                            const int so = 4 * q.own + kk;
+                            const int mxm = q.par ? m : (m + Lh - 1) % Lh;
+                            Jc[kk][0] = Js[so];
+                            Jc[kk][1] = Js[4 * ((cc * ROWS + r) * W) + mxm];
+                            Jc[kk][2] = Js[LB + so];
+                            Jc[kk][3] = Js[LB + 4 * ((cc * ROWS + rym) * W) + m];
+                            Jc[kk][4] = Js[2 * LB + so];
+                            Jc[kk][5] = Js[2 * LB + 4 * ((cc * ROWS + rzm) * W) + m];
+                        }
+                    }
+                    // the same couplings as packed pairs (sites 0,1 and 2,3); the x
+                    // pair is ordered as (aligned word xa, shifted word xs), so the
+                    // lattice loop needs no select on the row parity
+                    #pragma unroll
+                    for (int n = 0; n < 6; ++n) {
+                        Jp[0][n] = pack2(Jc[0][n], Jc[1][n]);
+                        Jp[1][n] = pack2(Jc[2][n], Jc[3][n]);
+                    }
+                    if (RULE != PTHR_HEATBATH && q.par) {
+    #pragma unroll
+                        for (int h = 0; h < 2; ++h) {
+                            const f2 t = Jp[h][0];
+                            Jp[h][0] = Jp[h][1];
+                            Jp[h][1] = t;
+                        }
+                    }
+}
+
+// A group's word and its six neighbour words (x aligned and shifted).
+struct Neighbours { uint32_t own, xa, xs, yp, ym, zp, zm; };
+__device__ __forceinline__ Neighbours group_words(const uint32_t *S, const GroupGeo &q) {
+    return Neighbours{S[q.own], S[q.xa], __byte_perm(S[q.wA], S[q.wB], q.selx), S[q.yp], S[q.ym], S[q.zp], S[q.zm]};
+}
+
+// Flip mask (bit 7 of every byte to flip) of one group of one lattice: tb =
+// -2 log2(e) / T, rw the group's random words; sel: the MicSA walker's word.
+template <int L, int RULE>
+__device__ __forceinline__ uint32_t group_flips(const Neighbours &nb, const f2 (&Jp)[2][6], float tb,
+                                                const uint32_t (&rw)[4], int sel, int par, uint32_t vmask) {
+    const uint32_t own = nb.own;
+    uint32_t fm = 0u;
+    if (RULE == PTHR_HEATBATH) {
+        const uint32_t wxp = par ? nb.xs : nb.xa, wxm = par ? nb.xa : nb.xs;
+        float Jc[4][6];
+#pragma unroll
+        for (int n = 0; n < 6; ++n) {
+            unpack2(Jp[0][n], Jc[0][n], Jc[1][n]);
+            unpack2(Jp[1][n], Jc[2][n], Jc[3][n]);
+        }
+#pragma unroll
+        for (int kk = 0; kk < 4; ++kk) {
+            const float si = spinf(own, kk);
+            float h = Jc[kk][0] * spinf(wxp, kk);
+            h = fmaf(Jc[kk][1], spinf(wxm, kk), h);
+            h = fmaf(Jc[kk][2], spinf(nb.yp, kk), h);
+            h = fmaf(Jc[kk][3], spinf(nb.ym, kk), h);
+            h = fmaf(Jc[kk][4], spinf(nb.zp, kk), h);
+            h = fmaf(Jc[kk][5], spinf(nb.zm, kk), h);
+            const float u = uniform24f(rw[kk]);
+            const float p_up = __frcp_rn(1.f + fast_exp2(tb * h));
+            const bool flip = (u < p_up) != (si > 0.f);
+            fm |= flip ? (0x80u << (8 * kk)) : 0u;
+        }
+        return fm & vmask;
+    }
+    // t = sum_j J_ij s_i s_j (packed): bytes 0x3F where s_i s_j = +1, 0xBF where -1
+    const uint32_t X = 0x3F3F3F3Fu;
+    const uint32_t pxa = own ^ nb.xa ^ X, pxs = own ^ nb.xs ^ X;
+    const uint32_t pyp = own ^ nb.yp ^ X, pym = own ^ nb.ym ^ X;
+    const uint32_t pzp = own ^ nb.zp ^ X, pzm = own ^ nb.zm ^ X;
+    f2 tt[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        tt[h] = mul2(Jp[h][0], spin_pair(pxa, h));
+        tt[h] = fma2(Jp[h][1], spin_pair(pxs, h), tt[h]);
+        tt[h] = fma2(Jp[h][2], spin_pair(pyp, h), tt[h]);
+        tt[h] = fma2(Jp[h][3], spin_pair(pym, h), tt[h]);
+        tt[h] = fma2(Jp[h][4], spin_pair(pzp, h), tt[h]);
+        tt[h] = fma2(Jp[h][5], spin_pair(pzm, h), tt[h]);
+    }
+    if (RULE == PTHR_MICSA) {
+        // one walker per (lattice, group, colour pass) with energy -T ln u;
+        // site kk flips iff u < 2^(tb y), y = D + t_kk, D the share already
+        // taken by this pass's flips (in units of t = Delta E / 2), then D = y
+        float tv[4];
+        unpack2(tt[0], tv[0], tv[1]);
+        unpack2(tt[1], tv[2], tv[3]);
+        const uint32_t wsel = sel == 0 ? rw[0] : (sel == 1 ? rw[1] : (sel == 2 ? rw[2] : rw[3]));
+        const float uw = uniform24f(wsel);
+        float D = 0.f;
+#pragma unroll
+        for (int kk = 0; kk < 4; ++kk) {
+            const float y = D + tv[kk];
+            if (uw < fast_exp2(tb * y)) {
+                D = y;
+                fm |= 0x80u << (8 * kk);
+            }
+        }
+        return fm & vmask;
+    }
+    float dv[4];
+    const f2 tb2 = pack2(tb, tb);
+    const f2 sc2 = pack2(5.9604644775390625e-08f, 5.9604644775390625e-08f);
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        float y0, y1;
+        unpack2(mul2(tb2, tt[h]), y0, y1);
+        const f2 negp = pack2(-fast_exp2(y0), -fast_exp2(y1));
+        // u - p < 0  <=>  accept (u = (x >> 8) 2^-24, exact)
+        const f2 u2 = pack2(__uint2float_rz(rw[2 * h] >> 8), __uint2float_rz(rw[2 * h + 1] >> 8));
+        unpack2(fma2(u2, sc2, negp), dv[2 * h], dv[2 * h + 1]);
+    }
+    // sign byte of each difference -> byte kk of the mask
+    const uint32_t lo = __byte_perm(__float_as_uint(dv[0]), __float_as_uint(dv[1]), 0x0073u);
+    const uint32_t hi = __byte_perm(__float_as_uint(dv[2]), __float_as_uint(dv[3]), 0x7300u);
+    return __byte_perm(lo, hi, 0x7610u) & vmask;
+}
+
 // Sums w and f over the lanes of this warp that share this thread's lattice
 // lane (a contiguous run of lanes: group index g0 within a lane of Gt
 // groups); the run's first lane (lane 0 or g0 == 0) holds the result.  nl =
@@ -243,7 +404,7 @@ struct SweepBounds {
 // One block of the sweep launch: block `bid` of the launch described by a,
 // dynamic shared memory at smem.  Threads past the block's lattice lanes
 // (a launch shared with larger shapes) take part in the barriers only.
-template <int L, int RULE, int KT>
+template <int L, int RULE, int KT, bool MAY_HOIST = true>
 __device__ __forceinline__ void sweep_block(const SweepArgs &a, int bid, unsigned char *smem) {
     using Gm = Geom<L>;
     constexpr int W = Gm::W, ROWS = Gm::ROWS, Lh = Gm::Lh, G = Gm::G;
@@ -455,12 +616,80 @@ __device__ __forceinline__ void sweep_block(const SweepArgs &a, int bid, unsigne
     // one group per colour (G <= 512): its geometry in both colours, once
     // (not where two blocks share an SM: there the registers are short)
     constexpr bool ONE_G = G <= 512 && SweepBounds<L, RULE>::min_blocks == 1;
+    constexpr bool HOIST = MAY_HOIST && G <= 512 && KT <= HOIST_KT;
     GroupGeo qc0{}, qc1{};
-    if (ONE_G) {
+    if (ONE_G || HOIST) {
         qc0 = group_geo<L>(g0, 0);
         qc1 = group_geo<L>(g0, 1);
     }
-    for (int sw = 0; sw < nsw; ++sw) {
+    // Few lattices per thread: the couplings of both colours stay in registers
+    // for all sweeps (loading and pairing a group's 24 couplings costs as much
+    // as updating one lattice: at L = 16 a half-sweep of a 512-thread block
+    // takes about 900 + 775 KT cycles with them in shared memory), and a
+    // half-sweep's random words are drawn before the barrier of the one before,
+    // since they do not depend on spins.  More than four lattices per thread
+    // would spill (48 coupling registers of 128).  240-sweep reservoir
+    // launches with four lattices per block: L = 16, 64 samples 1.62 ms (2.05
+    // ms); L = 4, one sample, KT = 1: 61 us (137 us).
+    if (HOIST) {
+        f2 Jr[2][2][6];
+        sweep_couplings<L, RULE>(Js, qc0, g0, 0, Jr[0]);
+        sweep_couplings<L, RULE>(Js, qc1, g0, 1, Jr[1]);
+        const uint32_t vmask = valid_mask<L>(g0 % W);
+        uint32_t ahi, alo;
+        mul_wide(0xD2511F53u, (uint32_t)g0, ahi, alo);
+        uint32_t c3 = (RULE == PTHR_MICSA ? TAG_MICSA : TAG_SWEEP) | ((uint32_t)sweep_base << 9);
+        uint4 lr[KT];
+        u4 rnd[KT];
+#pragma unroll
+        for (int jj = 0; jj < KT; ++jj) lr[jj] = s_lr[min(kbase + jj, K - 1)];
+        const auto draw = [&](u4 (&w)[KT]) {
+            const SweepRng rng = sweep_rng(ahi, alo, rng_elo, c3, rk0, rk1);
+#pragma unroll
+            for (int jj = 0; jj < KT; ++jj) {
+                if (RULE != PTHR_MICSA || jj == 0 || ((e0 + kbase + jj) & 3) == 0)
+                    w[jj] = philox10_sweep(lr[jj].x, lr[jj].y, rng, rk0, rk1);
+                else
+                    w[jj] = w[jj > 0 ? jj - 1 : 0];
+            }
+        };
+        draw(rnd);
+        for (int sw = 0; sw < nsw; ++sw) {
+#pragma unroll
+            for (int c = 0; c < 2; ++c) {
+                const GroupGeo &q = c ? qc1 : qc0;
+                // with one or two lattices the next words are drawn between
+                // this half-sweep's loads and their use (two serial chains
+                // side by side), else after it (the words of both would spill)
+                Neighbours nb[KT];
+                u4 next[KT];
+                c3 += 0x100u;                        // colour 1, then the next sweep's colour 0
+                if (KT <= 2) {
+#pragma unroll
+                    for (int jj = 0; jj < KT; ++jj) nb[jj] = group_words(Ss + min(kbase + jj, K - 1) * LW, q);
+                    draw(next);
+                }
+#pragma unroll
+                for (int jj = 0; jj < KT; ++jj) {
+                    if (KT > 2) {
+                        if (kbase + jj >= K) break;
+                        nb[jj] = group_words(Sb + jj * LW, q);
+                    }
+                    const uint32_t rw[4] = {rnd[jj].x, rnd[jj].y, rnd[jj].z, rnd[jj].w};
+                    const uint32_t fm = group_flips<L, RULE>(nb[jj], Jr[c], __uint_as_float(lr[jj].z), rw,
+                                                             (e0 + kbase + jj) & 3, q.par, vmask);
+                    if (kbase + jj < K) {
+                        Sb[jj * LW + q.own] = nb[jj].own ^ fm;
+                        nfl[jj] += __popc(fm);
+                    }
+                    if (KT <= 2) rnd[jj] = next[jj];
+                }
+                if (KT > 2) draw(rnd);
+                __syncthreads();
+            }
+        }
+    }
+    for (int sw = 0; !HOIST && sw < nsw; ++sw) {
         const uint32_t c3base = (RULE == PTHR_MICSA ? TAG_MICSA : TAG_SWEEP) | ((uint32_t)(sweep_base + sw) << 9);
         for (int c = 0; c < 2; ++c) {
             const uint32_t c3 = c3base | ((uint32_t)c << 8);
@@ -481,182 +710,24 @@ __device__ __forceinline__ void sweep_block(const SweepArgs &a, int bid, unsigne
                 uint32_t ahi, alo;
                 mul_wide(0xD2511F53u, (uint32_t)g, ahi, alo);
                 const SweepRng rng = sweep_rng(ahi, alo, rng_elo, c3, rk0, rk1);
-                const int j = g % W;
-                const int cc = c ^ 1;
-                const int r = g / W;
-                const int y = r % L, z = r / L;
-                const int rym = ((y + L - 1) % L) + L * z, rzm = y + L * ((z + L - 1) % L);
-                // couplings of the group's 4 sites: +x,-x,+y,-y,+z,-z
-                float Jc[4][6];
-                if (Gm::FULL) {
-                    // no row padding: the four sites' couplings of every
-                    // direction but -x are one aligned 16-byte load
-                    const float4 px = *reinterpret_cast<const float4 *>(Js + 4 * q.own);
-                    const float4 py = *reinterpret_cast<const float4 *>(Js + LB + 4 * q.own);
-                    const float4 pz = *reinterpret_cast<const float4 *>(Js + 2 * LB + 4 * q.own);
-                    const float4 my = *reinterpret_cast<const float4 *>(
-                        Js + LB + 4 * ((cc * ROWS + rym) * W) + 4 * j);
-                    const float4 mz = *reinterpret_cast<const float4 *>(
-                        Js + 2 * LB + 4 * ((cc * ROWS + rzm) * W) + 4 * j);
-                    const float vpx[4] = {px.x, px.y, px.z, px.w}, vpy[4] = {py.x, py.y, py.z, py.w};
-                    const float vpz[4] = {pz.x, pz.y, pz.z, pz.w}, vmy[4] = {my.x, my.y, my.z, my.w};
-                    const float vmz[4] = {mz.x, mz.y, mz.z, mz.w};
-#pragma unroll
-                    for (int kk = 0; kk < 4; ++kk) {
-                        const int m = 4 * j + kk;
-                        const int mxm = q.par ? m : (m + Lh - 1) % Lh;
-                        Jc[kk][0] = vpx[kk];
-                        Jc[kk][1] = Js[4 * ((cc * ROWS + r) * W) + mxm];
-                        Jc[kk][2] = vpy[kk];
-                        Jc[kk][3] = vmy[kk];
-                        Jc[kk][4] = vpz[kk];
-                        Jc[kk][5] = vmz[kk];
-                    }
-                } else {
-#pragma unroll
-                    for (int kk = 0; kk < 4; ++kk) {
-                        int m = 4 * j + kk;
-                        if (m >= Lh) m = Lh - 1;
-                        const int so = 4 * q.own + kk;
-                        const int mxm = q.par ? m : (m + Lh - 1) % Lh;
-                        Jc[kk][0] = Js[so];
-                        Jc[kk][1] = Js[4 * ((cc * ROWS + r) * W) + mxm];
-                        Jc[kk][2] = Js[LB + so];
-                        Jc[kk][3] = Js[LB + 4 * ((cc * ROWS + rym) * W) + m];
-                        Jc[kk][4] = Js[2 * LB + so];
-                        Jc[kk][5] = Js[2 * LB + 4 * ((cc * ROWS + rzm) * W) + m];
-                    }
-                }
-                // the same couplings as packed pairs (sites 0,1 and 2,3); the x
-                // pair is ordered as (aligned word xa, shifted word xs), so the
-                // lattice loop needs no select on the row parity
                 f2 Jp[2][6];
-#pragma unroll
-                for (int n = 0; n < 6; ++n) {
-                    Jp[0][n] = pack2(Jc[0][n], Jc[1][n]);
-                    Jp[1][n] = pack2(Jc[2][n], Jc[3][n]);
-                }
-                if (q.par) {
-#pragma unroll
-                    for (int h = 0; h < 2; ++h) {
-                        const f2 t = Jp[h][0];
-                        Jp[h][0] = Jp[h][1];
-                        Jp[h][1] = t;
-                    }
-                }
-                // flip-mask bits of the real sites of this group
-                uint32_t vmask = 0x80808080u;
-                if (!Gm::FULL) {
-                    const int nv = Lh - 4 * j;
-                    vmask = nv >= 4 ? 0x80808080u : (0x80808080u >> (8 * (4 - nv)));
-                }
-                u4 walker_rnd{};       // MicSA: one Philox call serves four positions
+                sweep_couplings<L, RULE>(Js, q, g, c, Jp);
+                const uint32_t vmask = valid_mask<L>(g % W);
+                u4 rnd{};
 #pragma unroll
                 for (int jj = 0; jj < KT; ++jj) {
                     const int k = kbase + jj;
                     if (k >= K) break;
                     uint32_t *S = Sb + jj * LW;
-                    const uint32_t own = S[q.own];
-                    const uint32_t xa = S[q.xa];
-                    const uint32_t xs = __byte_perm(S[q.wA], S[q.wB], q.selx);
-                    const uint32_t wyp = S[q.yp], wym = S[q.ym], wzp = S[q.zp], wzm = S[q.zm];
+                    const Neighbours nb = group_words(S, q);
                     const uint4 lr = s_lr[k];
-                    u4 rnd;
-                    if (RULE == PTHR_MICSA) {
-                        if (jj == 0 || ((e0 + k) & 3) == 0)
-                            walker_rnd = philox10_sweep(lr.x, lr.y, rng, rk0, rk1);
-                        rnd = walker_rnd;
-                    } else {
+                    // MicSA: one Philox call serves four positions
+                    if (RULE != PTHR_MICSA || jj == 0 || ((e0 + k) & 3) == 0)
                         rnd = philox10_sweep(lr.x, lr.y, rng, rk0, rk1);
-                    }
                     const uint32_t rw[4] = {rnd.x, rnd.y, rnd.z, rnd.w};
-                    const float tb = __uint_as_float(lr.z);
-                    uint32_t fm;
-                    if (RULE == PTHR_MICSA) {
-                        // one walker per (lattice, group, colour pass) with
-                        // energy -T ln u; site kk flips iff u < 2^(tb y), y =
-                        // D + t_kk, D the share already taken by this pass's
-                        // flips (in units of t = Delta E / 2), then D = y
-                        const uint32_t X = 0x3F3F3F3Fu;
-                        const uint32_t pxa = own ^ xa ^ X, pxs = own ^ xs ^ X;
-                        const uint32_t pyp = own ^ wyp ^ X, pym = own ^ wym ^ X;
-                        const uint32_t pzp = own ^ wzp ^ X, pzm = own ^ wzm ^ X;
-                        float tv[4];
-#pragma unroll
-                        for (int h = 0; h < 2; ++h) {
-                            f2 tt = mul2(Jp[h][0], spin_pair(pxa, h));
-                            tt = fma2(Jp[h][1], spin_pair(pxs, h), tt);
-                            tt = fma2(Jp[h][2], spin_pair(pyp, h), tt);
-                            tt = fma2(Jp[h][3], spin_pair(pym, h), tt);
-                            tt = fma2(Jp[h][4], spin_pair(pzp, h), tt);
-                            tt = fma2(Jp[h][5], spin_pair(pzm, h), tt);
-                            unpack2(tt, tv[2 * h], tv[2 * h + 1]);
-                        }
-                        const int sel = (e0 + k) & 3;
-                        const uint32_t wsel = sel == 0 ? rw[0] : (sel == 1 ? rw[1] : (sel == 2 ? rw[2] : rw[3]));
-                        const float uw = uniform24f(wsel);
-                        float D = 0.f;
-                        fm = 0u;
-#pragma unroll
-                        for (int kk = 0; kk < 4; ++kk) {
-                            const float y = D + tv[kk];
-                            const bool flip = uw < fast_exp2(tb * y);
-                            if (flip) {
-                                D = y;
-                                fm |= 0x80u << (8 * kk);
-                            }
-                        }
-                        fm &= vmask;
-                    } else if (RULE == PTHR_METROPOLIS) {
-                        // bytes 0x3F where s_i s_j = +1, 0xBF where -1
-                        const uint32_t X = 0x3F3F3F3Fu;
-                        const uint32_t pxa = own ^ xa ^ X, pxs = own ^ xs ^ X;
-                        const uint32_t pyp = own ^ wyp ^ X, pym = own ^ wym ^ X;
-                        const uint32_t pzp = own ^ wzp ^ X, pzm = own ^ wzm ^ X;
-                        float dv[4];
-                        const f2 tb2 = pack2(tb, tb);
-                        const f2 sc2 = pack2(5.9604644775390625e-08f, 5.9604644775390625e-08f);
-#pragma unroll
-                        for (int h = 0; h < 2; ++h) {
-                            // t = sum_j J_ij s_i s_j for sites 2h, 2h+1 (packed)
-                            f2 tt = mul2(Jp[h][0], spin_pair(pxa, h));
-                            tt = fma2(Jp[h][1], spin_pair(pxs, h), tt);
-                            tt = fma2(Jp[h][2], spin_pair(pyp, h), tt);
-                            tt = fma2(Jp[h][3], spin_pair(pym, h), tt);
-                            tt = fma2(Jp[h][4], spin_pair(pzp, h), tt);
-                            tt = fma2(Jp[h][5], spin_pair(pzm, h), tt);
-                            float y0, y1;
-                            unpack2(mul2(tb2, tt), y0, y1);
-                            const f2 negp = pack2(-fast_exp2(y0), -fast_exp2(y1));
-                            // u - p < 0  <=>  accept (u = (x >> 8) 2^-24, exact)
-                            const f2 u2 = pack2(__uint2float_rz(rw[2 * h] >> 8),
-                                                __uint2float_rz(rw[2 * h + 1] >> 8));
-                            unpack2(fma2(u2, sc2, negp), dv[2 * h], dv[2 * h + 1]);
-                        }
-                        // sign byte of each difference -> byte kk of the mask
-                        const uint32_t lo = __byte_perm(__float_as_uint(dv[0]), __float_as_uint(dv[1]), 0x0073u);
-                        const uint32_t hi = __byte_perm(__float_as_uint(dv[2]), __float_as_uint(dv[3]), 0x7300u);
-                        fm = __byte_perm(lo, hi, 0x7610u) & vmask;
-                    } else {
-                        fm = 0u;
-                        const uint32_t wxp = q.par ? xs : xa, wxm = q.par ? xa : xs;
-#pragma unroll
-                        for (int kk = 0; kk < 4; ++kk) {
-                            const float si = spinf(own, kk);
-                            float h = Jc[kk][0] * spinf(wxp, kk);
-                            h = fmaf(Jc[kk][1], spinf(wxm, kk), h);
-                            h = fmaf(Jc[kk][2], spinf(wyp, kk), h);
-                            h = fmaf(Jc[kk][3], spinf(wym, kk), h);
-                            h = fmaf(Jc[kk][4], spinf(wzp, kk), h);
-                            h = fmaf(Jc[kk][5], spinf(wzm, kk), h);
-                            const float u = uniform24f(rw[kk]);
-                            const float p_up = __frcp_rn(1.f + fast_exp2(tb * h));
-                            const bool flip = (u < p_up) != (si > 0.f);
-                            fm |= flip ? (0x80u << (8 * kk)) : 0u;
-                        }
-                        fm &= vmask;
-                    }
-                    S[q.own] = own ^ fm;
+                    const uint32_t fm = group_flips<L, RULE>(nb, Jp, __uint_as_float(lr.z), rw, (e0 + k) & 3, q.par,
+                                                             vmask);
+                    S[q.own] = nb.own ^ fm;
                     nfl[jj] += __popc(fm);
                 }
             }
