@@ -165,7 +165,7 @@ constexpr int GPU_SMS = 152;   // GB300
 // Kernel shapes.  Sweep: lattices per block K (PT / reservoir); Gt 4-site
 // groups per lattice lane (divides G, <= 512); P lattice lanes of KT
 // lattices each (KT one of the compiled variants); threads = P * Gt.
-struct SweepShape { int K_pt, K_res, Gt, P, KT, threads, pt_tasks, res_tasks; };
+struct SweepShape { int K_pt, K_res, Gt, P, KT, KT_res, threads, pt_tasks, res_tasks; };
 
 int default_k(const pthr_config *c, int total_entries) {
     const size_t lb = (size_t)lattice_words(c->L) * 4;
@@ -178,27 +178,36 @@ int default_k(const pthr_config *c, int total_entries) {
     return (int)k;
 }
 
+// Reservoir sweeps of a launch from which its reservoir blocks take their own
+// lattices per thread: the couplings of a small block are staged for fewer
+// lattices, which costs as much as 10 sweeps of 4 lattices gain (L = 16, 128
+// clones of 512 samples: 1 sweep 0.97 against 0.69 ms, 10 sweeps 3.73 against
+// 3.71 ms, 60 sweeps of 16 clones 2.47 against 3.04 ms).
+constexpr int RES_HOIST_SWEEPS = 16;
+
 // forced_kt > 0: lattices per thread fixed (the mixed-L group sweep compiles
 // one value per lattice size); the lattices per block then follow from it.
-// samples, res: the launch's samples and whether its long blocks are the
-// reservoir's (240 sweeps per EMCS against 10).
-SweepShape sweep_shape(const pthr_batch *b, int forced_kt, int samples, bool res) {
+// samples, res_sweeps: the launch's samples and reservoir sweeps; with any,
+// its long blocks are the reservoir's (240 sweeps per EMCS against 10).
+SweepShape sweep_shape(const pthr_batch *b, int forced_kt, int samples, int res_sweeps) {
     const pthr_config *c = &b->cfg;
+    const bool res = res_sweeps > 0;
     SweepShape sh{};
     const int npt = c->n_replicas * c->n_temps;
     const int nres = c->n_replicas * (c->n_res > 0 ? c->n_res : 1);
     sh.K_pt = default_k(c, npt);
     sh.K_res = default_k(c, nres);
     const int long_blocks = samples * (res ? (nres + sh.K_res - 1) / sh.K_res : (npt + sh.K_pt - 1) / sh.K_pt);
-    if (long_blocks < GPU_SMS && forced_kt == 0) {
+    const bool small = long_blocks < GPU_SMS && forced_kt == 0;
+    if (small) {
         // fewer long blocks than SMs: smaller blocks, and where a thread owns
         // one group of a colour (L <= 16) few enough lattices per thread to
         // keep its couplings in registers.  One EMCS alone / three batches on
         // three streams: L = 14, 20 samples 0.81 / 0.62 ms (16 lattices per
         // block: 3.05 / 1.02 ms); L = 18 MicSA, 24 samples 3.1 / 1.8 ms (5.5 /
         // 1.9 ms; 4 lattices: 2.2 / 2.0 ms); L = 16, 64 samples' reservoir
-        // sweeps 1.62 ms (3.1 ms).  From one block per SM on the larger blocks
-        // stay: their couplings serve more updates.
+        // sweeps 1.62 ms (3.1 ms).  From one block per SM on the PT clones'
+        // larger blocks stay: their couplings are staged for more updates.
         const bool one_group = sweep_groups_for(c->L) <= 512;
         const int most = one_group ? 4 : 8;
         if (sh.K_res > most) sh.K_res = most;
@@ -220,6 +229,23 @@ SweepShape sweep_shape(const pthr_batch *b, int forced_kt, int samples, bool res
     if (P0 < 1) P0 = 1;
     int opts[16];
     const int nopt = sweep_kt_options(c->L, c->update_rule, opts);
+    // Reservoir blocks of SWEEP_HOIST_KT lattices per thread with the couplings
+    // in registers beside PT blocks of more, where the caller's reservoir share
+    // fits the lanes: shorter blocks also fill the last wave (240-sweep EMCS,
+    // L = 16, 512 samples, three batches 13.56 -> 13.31 ms; 60 reservoir sweeps
+    // alone 3.04 -> 2.49 ms, heat bath 5.25 -> 4.00, MicSA 2.68 -> 2.28 ms).
+    bool res_hoist = res_sweeps >= RES_HOIST_SWEEPS && !small && Gt == G && opts[nopt - 1] > SWEEP_HOIST_KT &&
+                     (forced_kt > 0 || sweep_res_in_registers(c->L, c->update_rule));
+    if (b->tuning.res_lattices_per_block > 0) {
+        if (sh.K_res > P0 * SWEEP_HOIST_KT) res_hoist = false;
+    } else if (res_hoist && forced_kt == 0 && b->tuning.sweep_threads <= 0) {
+        // no more lanes than the reservoir's lattices fill, but four warps (60
+        // reservoir sweeps of 2048 samples: L = 8 1.65 -> 1.22 ms, L = 6 1.65 ->
+        // 0.96 ms against half of the lanes idle)
+        int lanes = (sh.K_res + SWEEP_HOIST_KT - 1) / SWEEP_HOIST_KT;
+        if (lanes * Gt < 128) lanes = (128 + Gt - 1) / Gt;
+        if (P0 > lanes) P0 = lanes;
+    }
     int Kmax = sh.K_pt > sh.K_res ? sh.K_pt : sh.K_res;
     if (P0 > Kmax) P0 = Kmax;
     const int need = (Kmax + P0 - 1) / P0;
@@ -233,7 +259,19 @@ SweepShape sweep_shape(const pthr_batch *b, int forced_kt, int samples, bool res
         Kmax = sh.K_pt > sh.K_res ? sh.K_pt : sh.K_res;
     }
     sh.KT = KT;
+    sh.KT_res = KT;
     sh.P = (Kmax + KT - 1) / KT;
+    if (res_hoist && KT > SWEEP_HOIST_KT) {
+        sh.KT_res = SWEEP_HOIST_KT;
+        if (sh.K_res > P0 * SWEEP_HOIST_KT) sh.K_res = P0 * SWEEP_HOIST_KT;
+        if (b->tuning.res_lattices_per_block <= 0) {
+            const int tasks = (nres + sh.K_res - 1) / sh.K_res;
+            sh.K_res = (nres + tasks - 1) / tasks;       // blocks of equal length
+        }
+        const int P_res = (sh.K_res + SWEEP_HOIST_KT - 1) / SWEEP_HOIST_KT;
+        sh.P = (sh.K_pt + KT - 1) / KT;
+        if (P_res > sh.P) sh.P = P_res;
+    }
     sh.threads = sh.P * Gt;
     sh.pt_tasks = (npt + sh.K_pt - 1) / sh.K_pt;
     sh.res_tasks = (nres + sh.K_res - 1) / sh.K_res;
@@ -246,7 +284,7 @@ struct SweepLaunch { SweepArgs a; int blocks, threads, KT; size_t smem; };
 pthr_status sweep_launch(pthr_batch *b, int n_pt, int n_res, int first, int count, int pretherm,
                          int forced_kt, SweepLaunch *out) {
     const pthr_config *c = &b->cfg;
-    SweepShape sh = sweep_shape(b, forced_kt, count, c->n_res > 0 && n_res > 0);
+    SweepShape sh = sweep_shape(b, forced_kt, count, c->n_res > 0 ? n_res : 0);
     SweepArgs a{};
     a.b = b->dev;
     a.n_pt_sweeps = n_pt;
@@ -263,6 +301,7 @@ pthr_status sweep_launch(pthr_batch *b, int n_pt, int n_res, int first, int coun
     a.sample_count = count;
     a.emcs_override = pretherm;
     a.Gt = sh.Gt;
+    a.KT_res = sh.KT_res;
     out->a = a;
     out->blocks = count * ((a.do_res ? sh.res_tasks : 0) + (a.do_pt ? sh.pt_tasks : 0));
     out->threads = sh.threads;
@@ -511,7 +550,7 @@ PTHR_API pthr_status pthr_set_tuning(pthr_batch *b, const pthr_tuning *t) {
         return fail(b, PTHR_E_INVAL, "tuning out of range");
     pthr_tuning old = b->tuning;
     b->tuning = nt;
-    SweepShape sh = sweep_shape(b, 0, b->cfg.n_samples, b->cfg.er_on != 0);
+    SweepShape sh = sweep_shape(b, 0, b->cfg.n_samples, b->cfg.er_on ? b->cfg.res_sweeps_per_emcs : 0);
     const size_t smem = sweep_smem_bytes_for(b->cfg.L, sh.K_pt > sh.K_res ? sh.K_pt : sh.K_res);
     if (smem > 220 * 1024) {
         b->tuning = old;
@@ -540,7 +579,7 @@ PTHR_API pthr_status pthr_set_update_rule(pthr_batch *b, int rule) {
 
 PTHR_API pthr_status pthr_get_tuning(const pthr_batch *b, pthr_tuning *t) {
     if (!b || !t) return fail(nullptr, PTHR_E_INVAL, "NULL argument");
-    SweepShape sh = sweep_shape(b, 0, b->cfg.n_samples, b->cfg.er_on != 0);
+    SweepShape sh = sweep_shape(b, 0, b->cfg.n_samples, b->cfg.er_on ? b->cfg.res_sweeps_per_emcs : 0);
     t->pt_lattices_per_block = sh.K_pt;
     t->res_lattices_per_block = sh.K_res;
     t->sweep_threads = sh.threads;

@@ -17,12 +17,18 @@ struct SweepArgs {
     int emcs_override;                   // 1: counter word PRETHERM_EMCS, sweep index
                                          //    from the sample's PRETH counter
     int Gt;                              // groups per lattice lane (divides G and threads)
+    int KT_res;                          // lattices per thread of the reservoir blocks: the
+                                         //    launch's own or SWEEP_HOIST_KT
 };
+// lattices per thread up to which the sweep keeps the couplings in registers
+// (where a thread owns one group of a colour)
+constexpr int SWEEP_HOIST_KT = 4;
 
 cudaError_t launch_sweep(const SweepArgs &a, int blocks, int threads, int KT, cudaStream_t st);
 size_t sweep_smem_bytes_for(int L, int K);
 int sweep_groups_for(int L);
 int sweep_max_k();
+bool sweep_res_in_registers(int L, int rule);      // sizes with reservoir blocks of SWEEP_HOIST_KT
 int sweep_kt_options(int L, int rule, int *out);   // compiled lattices-per-thread values
 
 // cluster.cu

@@ -18,6 +18,16 @@ int sweep_groups_for(int L) {
 
 int sweep_max_k() { return sweep_detail::MAXK; }
 
+bool sweep_res_in_registers(int L, int rule) {
+    using namespace sweep_detail;
+#define X(LL) if (L == LL) \
+        return rule == PTHR_HEATBATH ? res_in_registers<LL, PTHR_HEATBATH>() \
+               : rule == PTHR_MICSA  ? res_in_registers<LL, PTHR_MICSA>() : res_in_registers<LL, PTHR_METROPOLIS>();
+    PTHR_FOR_EACH_L(X)
+#undef X
+    return false;
+}
+
 // Lattices-per-thread values compiled for (L, rule), ascending.
 int sweep_kt_options(int L, int rule, int *out) {
     int n = 0;

@@ -33,7 +33,7 @@ template <int N>
 struct Const { static constexpr int value = N; };
 
 constexpr int MAXK = 64;   // lattices per block
-constexpr int HOIST_KT = 4;   // lattices per thread up to which the couplings stay in registers
+constexpr int HOIST_KT = SWEEP_HOIST_KT;
 
 // 32x32 -> 64-bit product as one wide multiply.
 __device__ __forceinline__ void mul_wide(uint32_t a, uint32_t b, uint32_t &hi, uint32_t &lo) {
@@ -904,10 +904,27 @@ __device__ __forceinline__ void sweep_block(const SweepArgs &a, int bid, unsigne
     }
 }
 
+// Whether the launch's reservoir blocks may run HOIST_KT lattices per thread
+// beside PT blocks of more: where a thread owns one group of a colour and no
+// second block shares the SM (there, L = 12 Metropolis, the registers of both
+// paths spill: one-sweep launches of 1024 samples 2.4% slower).
+template <int L, int RULE>
+__host__ __device__ constexpr bool res_in_registers() { return Geom<L>::G <= 512 && SweepBounds<L, RULE>::min_blocks == 1; }
+
+__device__ __forceinline__ bool res_block_in_registers(const SweepArgs &a, int bid) {
+    return a.KT_res == HOIST_KT && a.do_res && bid < a.sample_count * a.res_tasks;
+}
+
 template <int L, int RULE, int KT>
 __global__ void __launch_bounds__(SweepBounds<L, RULE>::threads, SweepBounds<L, RULE>::min_blocks)
 sweep_kernel(SweepArgs a) {
     extern __shared__ __align__(16) unsigned char smem[];
+    if constexpr (KT > HOIST_KT && res_in_registers<L, RULE>()) {
+        if (res_block_in_registers(a, blockIdx.x)) {
+            sweep_block<L, RULE, HOIST_KT>(a, blockIdx.x, smem);
+            return;
+        }
+    }
     sweep_block<L, RULE, KT>(a, blockIdx.x, smem);
 }
 
