@@ -195,68 +195,68 @@ template <int L, int RULE>
 __device__ __forceinline__ void sweep_couplings(const float *Js, const GroupGeo &q, int g, int c, f2 (&Jp)[2][6]) {
     using Gm = Geom<L>;
     constexpr int W = Gm::W, ROWS = Gm::ROWS, Lh = Gm::Lh, LB = Gm::LAT_BYTES;
-                    const int j = g % W;
-                    const int cc = c ^ 1;
-                    const int r = g / W;
-                    const int y = r % L, z = r / L;
-                    const int rym = ((y + L - 1) % L) + L * z, rzm = y + L * ((z + L - 1) % L);
-                    // couplings of the group's 4 sites: +x,-x,+y,-y,+z,-z
-                    float Jc[4][6];
-                    if (Gm::FULL) {
-                        // no row padding: the four sites' couplings of every
-                        // direction but -x are one aligned 16-byte load
-                        const float4 px = *reinterpret_cast<const float4 *>(Js + 4 * q.own);
-                        const float4 py = *reinterpret_cast<const float4 *>(Js + LB + 4 * q.own);
-                        const float4 pz = *reinterpret_cast<const float4 *>(Js + 2 * LB + 4 * q.own);
-                        const float4 my = *reinterpret_cast<const float4 *>(
-                            Js + LB + 4 * ((cc * ROWS + rym) * W) + 4 * j);
-                        const float4 mz = *reinterpret_cast<const float4 *>(
-                            Js + 2 * LB + 4 * ((cc * ROWS + rzm) * W) + 4 * j);
-                        const float vpx[4] = {px.x, px.y, px.z, px.w}, vpy[4] = {py.x, py.y, py.z, py.w};
-                        const float vpz[4] = {pz.x, pz.y, pz.z, pz.w}, vmy[4] = {my.x, my.y, my.z, my.w};
-                        const float vmz[4] = {mz.x, mz.y, mz.z, mz.w};
-    #pragma unroll
-                        for (int kk = 0; kk < 4; ++kk) {
-                            const int m = 4 * j + kk;
-                            const int mxm = q.par ? m : (m + Lh - 1) % Lh;
-                            Jc[kk][0] = vpx[kk];
-                            Jc[kk][1] = Js[4 * ((cc * ROWS + r) * W) + mxm];
-                            Jc[kk][2] = vpy[kk];
-                            Jc[kk][3] = vmy[kk];
-                            Jc[kk][4] = vpz[kk];
-                            Jc[kk][5] = vmz[kk];
-                        }
-                    } else {
-    #pragma unroll
-                        for (int kk = 0; kk < 4; ++kk) {
-                            int m = 4 * j + kk;
-                            if (m >= Lh) m = Lh - 1;
-                            const int so = 4 * q.own + kk;
-                            const int mxm = q.par ? m : (m + Lh - 1) % Lh;
-                            Jc[kk][0] = Js[so];
-                            Jc[kk][1] = Js[4 * ((cc * ROWS + r) * W) + mxm];
-                            Jc[kk][2] = Js[LB + so];
-                            Jc[kk][3] = Js[LB + 4 * ((cc * ROWS + rym) * W) + m];
-                            Jc[kk][4] = Js[2 * LB + so];
-                            Jc[kk][5] = Js[2 * LB + 4 * ((cc * ROWS + rzm) * W) + m];
-                        }
-                    }
-                    // the same couplings as packed pairs (sites 0,1 and 2,3); the x
-                    // pair is ordered as (aligned word xa, shifted word xs), so the
-                    // lattice loop needs no select on the row parity
-                    #pragma unroll
-                    for (int n = 0; n < 6; ++n) {
-                        Jp[0][n] = pack2(Jc[0][n], Jc[1][n]);
-                        Jp[1][n] = pack2(Jc[2][n], Jc[3][n]);
-                    }
-                    if (RULE != PTHR_HEATBATH && q.par) {
-    #pragma unroll
-                        for (int h = 0; h < 2; ++h) {
-                            const f2 t = Jp[h][0];
-                            Jp[h][0] = Jp[h][1];
-                            Jp[h][1] = t;
-                        }
-                    }
+    const int j = g % W;
+    const int cc = c ^ 1;
+    const int r = g / W;
+    const int y = r % L, z = r / L;
+    const int rym = ((y + L - 1) % L) + L * z, rzm = y + L * ((z + L - 1) % L);
+    // couplings of the group's 4 sites: +x,-x,+y,-y,+z,-z
+    float Jc[4][6];
+    if (Gm::FULL) {
+        // no row padding: the four sites' couplings of every
+        // direction but -x are one aligned 16-byte load
+        const float4 px = *reinterpret_cast<const float4 *>(Js + 4 * q.own);
+        const float4 py = *reinterpret_cast<const float4 *>(Js + LB + 4 * q.own);
+        const float4 pz = *reinterpret_cast<const float4 *>(Js + 2 * LB + 4 * q.own);
+        const float4 my = *reinterpret_cast<const float4 *>(
+            Js + LB + 4 * ((cc * ROWS + rym) * W) + 4 * j);
+        const float4 mz = *reinterpret_cast<const float4 *>(
+            Js + 2 * LB + 4 * ((cc * ROWS + rzm) * W) + 4 * j);
+        const float vpx[4] = {px.x, px.y, px.z, px.w}, vpy[4] = {py.x, py.y, py.z, py.w};
+        const float vpz[4] = {pz.x, pz.y, pz.z, pz.w}, vmy[4] = {my.x, my.y, my.z, my.w};
+        const float vmz[4] = {mz.x, mz.y, mz.z, mz.w};
+#pragma unroll
+        for (int kk = 0; kk < 4; ++kk) {
+            const int m = 4 * j + kk;
+            const int mxm = q.par ? m : (m + Lh - 1) % Lh;
+            Jc[kk][0] = vpx[kk];
+            Jc[kk][1] = Js[4 * ((cc * ROWS + r) * W) + mxm];
+            Jc[kk][2] = vpy[kk];
+            Jc[kk][3] = vmy[kk];
+            Jc[kk][4] = vpz[kk];
+            Jc[kk][5] = vmz[kk];
+        }
+    } else {
+#pragma unroll
+        for (int kk = 0; kk < 4; ++kk) {
+            int m = 4 * j + kk;
+            if (m >= Lh) m = Lh - 1;
+            const int so = 4 * q.own + kk;
+            const int mxm = q.par ? m : (m + Lh - 1) % Lh;
+            Jc[kk][0] = Js[so];
+            Jc[kk][1] = Js[4 * ((cc * ROWS + r) * W) + mxm];
+            Jc[kk][2] = Js[LB + so];
+            Jc[kk][3] = Js[LB + 4 * ((cc * ROWS + rym) * W) + m];
+            Jc[kk][4] = Js[2 * LB + so];
+            Jc[kk][5] = Js[2 * LB + 4 * ((cc * ROWS + rzm) * W) + m];
+        }
+    }
+    // the same couplings as packed pairs (sites 0,1 and 2,3); the x
+    // pair is ordered as (aligned word xa, shifted word xs), so the
+    // lattice loop needs no select on the row parity
+#pragma unroll
+    for (int n = 0; n < 6; ++n) {
+        Jp[0][n] = pack2(Jc[0][n], Jc[1][n]);
+        Jp[1][n] = pack2(Jc[2][n], Jc[3][n]);
+    }
+    if (RULE != PTHR_HEATBATH && q.par) {
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const f2 t = Jp[h][0];
+            Jp[h][0] = Jp[h][1];
+            Jp[h][1] = t;
+        }
+    }
 }
 
 // A group's word and its six neighbour words (x aligned and shifted).
@@ -775,8 +775,9 @@ __device__ __forceinline__ void sweep_block(const SweepArgs &a, int bid, unsigne
         // hand, with its sign turned where the site flipped.  Only a launch
         // without sweeps computes the fields.  (A pass of its own over the
         // colour-0 sites after every launch: one-sweep launches of L = 12, 1024
-        // samples 560 us against 502 us, L = 8, 256 samples 29.7 against 27.3.)  With the couplings scaled by 2^18 every t_i is an integer
-        // below 2^24 in FP32; the sums run in integers.
+        // samples 560 us against 502 us, L = 8, 256 samples 29.7 against 27.3.)
+        // With the couplings scaled by 2^18 every t_i is an integer below 2^24
+        // in FP32; the sums run in integers.
         if (nsw == 0) {
             for (int gi = 0; gi < GP; ++gi) {
                 const int g = g0 + gi * Gt;

@@ -2,7 +2,9 @@
 // Lattices per thread KT times lattice lanes P is the lattices per block K;
 // the largest KT per L follows the shared-memory bound on K (L = 12 stops at
 // 16, the largest that fits two blocks per SM without spilling).  Variants of
-// up to four keep the couplings in registers; launches of few blocks use them.
+// up to four keep the couplings in registers; launches of few blocks use them,
+// and the reservoir's blocks of larger launches run four inside the variants
+// of more.
 #pragma once
 
 #include <cuda_runtime.h>
