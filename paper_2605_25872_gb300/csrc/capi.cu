@@ -233,7 +233,8 @@ SweepShape sweep_shape(const pthr_batch *b, int forced_kt, int samples, int res_
     // in registers beside PT blocks of more, where the caller's reservoir share
     // fits the lanes: shorter blocks also fill the last wave (240-sweep EMCS,
     // L = 16, 512 samples, three batches 13.56 -> 13.31 ms; 60 reservoir sweeps
-    // alone 3.04 -> 2.49 ms, heat bath 5.25 -> 4.00, MicSA 2.68 -> 2.28 ms).
+    // alone 3.04 -> 2.49 ms; 10 PT and 240 reservoir sweeps with the heat bath
+    // 23.8 -> 21.6 ms, MicSA at L = 10, 1024 samples 14.7 -> 10.8 ms).
     bool res_hoist = res_sweeps >= RES_HOIST_SWEEPS && !small && Gt == G && opts[nopt - 1] > SWEEP_HOIST_KT &&
                      (forced_kt > 0 || sweep_res_in_registers(c->L, c->update_rule));
     if (b->tuning.res_lattices_per_block > 0) {

@@ -908,9 +908,16 @@ __device__ __forceinline__ void sweep_block(const SweepArgs &a, int bid, unsigne
 // Whether the launch's reservoir blocks may run HOIST_KT lattices per thread
 // beside PT blocks of more: where a thread owns one group of a colour and no
 // second block shares the SM (there, L = 12 Metropolis, the registers of both
-// paths spill: one-sweep launches of 1024 samples 2.4% slower).
+// paths spill: one-sweep launches of 1024 samples 2.4% slower).  Not for MicSA
+// on 512 groups (L = 16: one draw serves four lattices and the couplings come
+// by 16-byte loads; 10 PT and 240 reservoir sweeps of 512 samples 11.54 ms
+// with the one form, 11.89 ms with both; L = 14, 256 samples 6.65 and 6.61,
+// L = 10, 1024 samples 14.66 and 10.81).
 template <int L, int RULE>
-__host__ __device__ constexpr bool res_in_registers() { return Geom<L>::G <= 512 && SweepBounds<L, RULE>::min_blocks == 1; }
+__host__ __device__ constexpr bool res_in_registers() {
+    return Geom<L>::G <= 512 && SweepBounds<L, RULE>::min_blocks == 1 &&
+           !(RULE == PTHR_MICSA && Geom<L>::G == 512);
+}
 
 __device__ __forceinline__ bool res_block_in_registers(const SweepArgs &a, int bid) {
     return a.KT_res == HOIST_KT && a.do_res && bid < a.sample_count * a.res_tasks;
