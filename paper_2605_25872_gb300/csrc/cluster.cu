@@ -424,24 +424,29 @@ __device__ __forceinline__ void finish_pair(const ClusterArgs &a, const PairItem
     const bool exact_E = ((off >> (sub * LN)) & (unsigned)((1ull << LN) - 1ull)) == 0u;
     double Ea = 0.0, Eb = 0.0;
     if (go && !exact_E && yl < L) {
-        float h = 0.f, l = 0.f, h2 = 0.f, l2 = 0.f;
         for (int z = 0; z < L; ++z) {
             const int r = y + L * z, ry = yp + L * z, rz = y + L * ((z + 1) % L);
             const uint32_t ar = as[r] ^ Fs[r], ay = as[ry] ^ Fs[ry], az = as[rz] ^ Fs[rz];
             const uint32_t br = ar ^ qs[r], by = ay ^ qs[ry], bz = az ^ qs[rz];
             const uint32_t na[3] = {ar ^ rot_next<L>(ar), ar ^ ay, ar ^ az};
             const uint32_t nb[3] = {br ^ rot_next<L>(br), br ^ by, br ^ bz};
-            for (int x = 0; x < L; ++x) {
+            // FP32 pairs over half a row's bonds (at most 36 terms), added up
+            // in FP64: the low part of a sum over all of the lane's 3 L^2
+            // bonds would itself round (L = 24: 2e-14 of the energy, 2e-16 so)
+            for (int x0 = 0; x0 < L; x0 += L / 2) {
+                float h = 0.f, l = 0.f, h2 = 0.f, l2 = 0.f;
+                for (int x = x0; x < x0 + L / 2; ++x) {
 #pragma unroll
-                for (int d = 0; d < 3; ++d) {
-                    const float j = __ldg(J + d * V + L * r + x);
-                    two_sum_acc(h, l, ((na[d] >> x) & 1u) ? -j : j);
-                    two_sum_acc(h2, l2, ((nb[d] >> x) & 1u) ? -j : j);
+                    for (int d = 0; d < 3; ++d) {
+                        const float j = __ldg(J + d * V + L * r + x);
+                        two_sum_acc(h, l, ((na[d] >> x) & 1u) ? -j : j);
+                        two_sum_acc(h2, l2, ((nb[d] >> x) & 1u) ? -j : j);
+                    }
                 }
+                Ea += (double)h + (double)l;
+                Eb += (double)h2 + (double)l2;
             }
         }
-        Ea = (double)h + (double)l;
-        Eb = (double)h2 + (double)l2;
     }
     for (int o = LN / 2; o > 0; o >>= 1) {
         dE += __shfl_xor_sync(FULLW, dE, o);
