@@ -140,6 +140,15 @@ __device__ __forceinline__ uint32_t word_flips(uint32_t v, int j) {
     return (((v >> (8 * j)) & 0x55u) * 0x02082080u) & 0x80808080u;
 }
 
+// 2^18 J (negated: -2^18 J) as an integer (adding 1.5 2^23 rounds to one); bad
+// is set where the integer does not give J back.  By value: a zero of either
+// sign is on the grid.
+__device__ __forceinline__ int bond_int(float j, bool negated, uint32_t &bad) {
+    const int v = __float_as_int(fmaf(j, 262144.f, 12582912.f)) - 0x4B400000;
+    bad |= (float)v * 3.814697265625e-06f != j;
+    return negated ? -v : v;
+}
+
 // ------------------------------------------------------------ items
 struct PairItem {
     bool live;
@@ -407,12 +416,8 @@ __device__ __forceinline__ void finish_pair(const ClusterArgs &a, const PairItem
             for (int i = yl; i < listed; i += LN) {
                 const uint32_t e = list[i];
                 const uint32_t site = e & ((1u << SITE_BITS) - 1u), d = (e >> SITE_BITS) & 3u;
-                const float j = __uint_as_float(__float_as_uint(__ldg(J + d * V + site)) ^ ((e >> (SITE_BITS + 2)) << 31));
-                // J 2^18 as an integer (adding 1.5 2^23 rounds to one); it is
-                // J exactly iff the integer gives J back bit for bit
-                const int v = __float_as_int(fmaf(j, 262144.f, 12582912.f)) - 0x4B400000;
-                bad |= __float_as_uint((float)v * 3.814697265625e-06f) ^ __float_as_uint(j);
-                sum += v;                                // at most N / LN terms below 2^23
+                // (at most N / LN terms below 2^23)
+                sum += bond_int(__ldg(J + d * V + site), (e >> (SITE_BITS + 2)) != 0u, bad);
             }
             dE += sum;
             __syncwarp();

@@ -1,5 +1,6 @@
 """Energies after a cluster move for couplings other than Gaussian ones on the
-grid: wide-ranging float32 couplings (every clone's energy is recomputed)."""
+grid: wide-ranging float32 couplings (every clone's energy is recomputed) and
+diluted ones (zeros are on the grid: the energies are updated in integers)."""
 import math
 
 import numpy as np
@@ -62,3 +63,25 @@ def test_off_grid_energies_are_exact(L):
     assert moved.sum() >= 4
     for s, lat in np.argwhere(moved):
         assert E[s, lat] == energy(L, J[s], after[s, lat]), (s, lat)
+
+
+@pytest.mark.parametrize("zero", [0.0, -0.0])
+@pytest.mark.parametrize("L", [8, 14, 18])
+def test_zero_couplings_are_on_the_grid(L, zero):
+    # On the grid the move adds an exact difference to the resident energies:
+    # a shift planted in both clones' energies is still there afterwards, where
+    # a recomputation would drop it.
+    cfg = BatchConfig(L=L, n_samples=2, n_temps=6, t_min=0.2, t_max=0.8, n_replicas=2, n_res=0, er_on=False)
+    J = W.gaussian_couplings(L, 2, 80 + L)
+    J[np.random.Generator(np.random.PCG64(L)).random(J.shape) < 0.5] = zero
+    b = Batch(cfg, couplings=J, seeds=W.sample_seeds(W.SEED_BASE + 80 + L, 2))
+    b.import_spins(torch.from_numpy(domain_pairs(cfg, 81 + L)))
+    before = b.export_spins().cpu().numpy()
+    b.energies.add_(1024.0)
+    b.houdayer()
+    after = b.export_spins().cpu().numpy()
+    E = b.energies.cpu().numpy()
+    assert (before != after).any(-1).sum() >= 4
+    for s in range(2):
+        for lat in range(cfg.n_lat):
+            assert E[s, lat] == energy(L, J[s], after[s, lat]) + 1024.0, (s, lat)
