@@ -756,7 +756,7 @@ __device__ __forceinline__ void cluster_block(const ClusterArgs &a, int bid, uns
         // 90 cycles (on thermalised pairs four chains need 5% more row visits
         // than one, and a quarter of the serial steps)
         constexpr int CH = (L + 3) / 4;
-        bool more = true;
+        unsigned more = FULLW;                           // lanes with changes in the last pass
         for (int it = 0; more && it < 2 * cap; ++it) {
             uint32_t ch = 0;
             if ((it & 1) == 0) {
@@ -770,9 +770,10 @@ __device__ __forceinline__ void cluster_block(const ClusterArgs &a, int bid, uns
 #pragma unroll
                     for (int z = v; z < L; z += CH) ch |= flood_row<L>(f, m, ur, z, lp, lm);
             }
-            more = __any_sync(FULLW, ch != 0u);
+            more = __ballot_sync(FULLW, ch != 0u);
         }
-        if (more && act) ok = false;
+        // (of this pair: its neighbours in the warp may have converged)
+        if ((more >> (sub * LN)) & (unsigned)((1ull << LN) - 1ull)) ok = false;
         int size = 0;                                    // both clusters' sites, 16 bits each
 #pragma unroll
         for (int z = 0; z < L; ++z)
