@@ -239,7 +239,8 @@ PTHR_API pthr_status pthr_houdayer(pthr_batch *b);
 /* Canonical cluster labels (step (ii) without the flip) of every replica pair
  * at every temperature: out_device int32 [S][n_replicas/2][n_temps][V]
  * receives, for each site, the smallest site index of its cluster (the
- * connected component of {i ~ j : neighbours, q_i q_j > 0}, Sec. 3).
+ * connected component of {i ~ j : neighbours, q_i q_j > 0}, Sec. 3), or -1
+ * throughout a pair whose labelling hit its bound (PTHR_E_NOCONVERGE).
  * Diagnostic entry point; the spins are not changed. */
 PTHR_API pthr_status pthr_cluster_labels(pthr_batch *b, int32_t *out_device);
 

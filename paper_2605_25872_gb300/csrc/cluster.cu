@@ -345,7 +345,13 @@ __device__ __forceinline__ void finish_pair(const ClusterArgs &a, const PairItem
     uint32_t *B = b.spins + ((size_t)p.s * b.NLAT + p.lb) * b.lat_words;
     if (p.live && !ok && yl == 0) set_status(b.status, STATUS_NOCONVERGE);
     __syncwarp();
-    if (a.label_only) return;
+    if (a.label_only) {
+        if (p.live && !ok) {                             // no label rather than those of some clusters
+            int32_t *out = a.labels_out + ((size_t)(p.s * b.NPAIR + p.P) * b.NT + p.k) * V;
+            for (int i = yl; i < V; i += LN) out[i] = -1;
+        }
+        return;
+    }
     const bool go = p.live && ok;                        // the same for all lanes of the pair
 
     // ---- energies (Eq. (1)).  Only bonds with exactly one flipped end change:

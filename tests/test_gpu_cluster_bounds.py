@@ -57,3 +57,12 @@ def test_only_the_pairs_that_ran_out_stay_as_they_were():
             assert not cs[k].any()
             np.testing.assert_array_equal(out[[k, cfg.n_slot + k]], spins[0, [k, cfg.n_slot + k]])
             np.testing.assert_array_equal(b.energies.cpu().numpy()[0, [k, cfg.n_slot + k]], e[0, [k, cfg.n_slot + k]])
+
+
+def test_labels_of_a_pair_that_ran_out_are_absent():
+    cfg, b, spins = batch()
+    lab = b.cluster_labels().cpu().numpy()[0, 0]
+    assert b.poll(10000) == _lib.PTHR_E_NOCONVERGE
+    for k, form in enumerate(FORMS):
+        ref = O.cc_labels(L, spins[0, k], spins[0, cfg.n_slot + k])[0] if form == "star" else -1
+        np.testing.assert_array_equal(lab[k], ref if form == "star" else np.full(cfg.V, -1))
