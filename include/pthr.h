@@ -158,8 +158,9 @@ typedef struct {
     int pt_lattices_per_block;    /* lattices of one sample per sweep block, PT      */
     int res_lattices_per_block;   /* same for reservoir clones                       */
     int sweep_threads;            /* threads per sweep block (multiple of the work)  */
-    int cluster_threads;          /* threads per cluster-move block (<= 512; blocks
-                                     have at most 128)                               */
+    int cluster_threads;          /* threads per cluster-move block (<= 512): up to
+                                     128, blocks whose warps hold whole pairs; above,
+                                     one block per pair                              */
     int cluster_iter_cap;         /* 0: automatic bound 4V+64 on every labelling
                                      loop; a small value exercises the bounded-loop
                                      error path (PTHR_E_NOCONVERGE, spins unchanged) */

@@ -325,6 +325,28 @@ pthr_status do_sweep(pthr_batch *b, int n_pt, int n_res, int first, int count, i
     return PTHR_OK;
 }
 
+// Pairs below which a cluster launch gives each pair a block of its own: a
+// warp's floods are one serial chain that a small launch lasts as long as.
+// The line is about where the gain of one launch alone equals the loss of three
+// on streams of their own (thermalised; us per launch, block per pair / warps,
+// alone and of three): L = 8, 896 pairs 20 / 26 and 8.9 / 8.8, 1344 pairs 23 /
+// 26 and 12 / 9; L = 16, 448 pairs 37 / 56 and 24 / 19, 672 pairs 57 / 56 and
+// 32 / 20; L = 20, 448 pairs 71 / 111 and 46 / 45, 672 pairs 99 / 113 and 71 / 48.
+int cluster_pair_limit(int L) {
+    return L <= 8 ? 7 * GPU_SMS : (L <= 10 ? 4 * GPU_SMS : 7 * GPU_SMS / 2);
+}
+
+// Threads of a block per pair, 0: warps hold the pairs.  By default about eight
+// sites per thread; a caller's value above CLUSTER_MAX_THREADS asks for it.
+int pair_block_threads(const pthr_batch *b, int pairs) {
+    if (b->tuning.cluster_iter_cap > 0) return 0;
+    if (b->tuning.cluster_threads > 0)
+        return b->tuning.cluster_threads > CLUSTER_MAX_THREADS ? b->tuning.cluster_threads / 32 * 32 : 0;
+    if (pairs >= cluster_pair_limit(b->cfg.L)) return 0;
+    const int t = (b->cfg.L * b->cfg.L * b->cfg.L / 8 + 31) / 32 * 32;
+    return t <= CLUSTER_MAX_THREADS ? CLUSTER_MAX_THREADS + 32 : (t > 512 ? 512 : t);
+}
+
 // Threads per cluster-move block: whole warps, each with one to eight pairs
 // (larger requests run as blocks of CLUSTER_MAX_THREADS).  By default the
 // largest block that still gives every SM two: a warp works alone until the
@@ -353,6 +375,10 @@ pthr_status do_cluster(pthr_batch *b, int label_only, int32_t *labels) {
     a.label_only = label_only;
     a.labels_out = labels;
     a.iter_cap = b->tuning.cluster_iter_cap;
+    if (const int pair_threads = pair_block_threads(b, a.sample_count * a.b.NPAIR * a.b.n_acu)) {
+        CUDA_TRY(b, launch_cluster_pairs(a, pair_threads, b->stream), "cluster launch");
+        return PTHR_OK;
+    }
     const int threads = cluster_threads_of(b);
     if (cluster_smem_bytes_for(b->cfg.L, threads) > 200 * 1024)
         return fail(b, PTHR_E_INVAL, "cluster block does not fit in shared memory");
@@ -584,7 +610,8 @@ PTHR_API pthr_status pthr_get_tuning(const pthr_batch *b, pthr_tuning *t) {
     t->pt_lattices_per_block = sh.K_pt;
     t->res_lattices_per_block = sh.K_res;
     t->sweep_threads = sh.threads;
-    t->cluster_threads = cluster_threads_of(b);
+    t->cluster_threads = pair_block_threads(b, b->cfg.n_samples * b->dev.NPAIR * b->dev.n_acu);
+    if (t->cluster_threads == 0) t->cluster_threads = cluster_threads_of(b);
     t->cluster_iter_cap = b->tuning.cluster_iter_cap;
     return PTHR_OK;
 }

@@ -32,7 +32,8 @@
 // that it replaces: L = 12, 28672 pairs 203 us (611 us); L = 16, 18432 pairs
 // 247 us (887 us); L = 8, 5120 pairs 36 us (44 us); at a random start, where
 // clusters are many, 269 us (705 us) and 356 us (1000 us).  Launches of few
-// pairs last as long as one warp's chain: L = 14, 840 pairs 45 us (49 us).
+// pairs have a block each (pair_kernel); between the two, a launch lasts as
+// long as one warp's chain: L = 14, 840 pairs 45 us (49 us).
 #include "kernels.cuh"
 #include "bitrows.cuh"
 
@@ -70,16 +71,18 @@ constexpr size_t cluster_smem(int threads) {
 }
 
 // ------------------------------------------------------------ union-find
-__device__ __forceinline__ int find_root(volatile uint16_t *parent, int x, int cap, bool &ok,
+// Parent: 16 bits, or int where the memory allows it.
+template <typename Parent>
+__device__ __forceinline__ int find_root(volatile Parent *parent, int x, int cap, bool &ok,
                                          uint32_t *status, int V) {
     for (int it = 0; it < cap; ++it) {
         const int p = parent[x];
         if (p == x) return x;
 #ifdef PTHR_DEBUG
-        if (!PTHR_DCHECK(status, p >= 0 && p < V && parent[p] < V)) { ok = false; return x; }
+        if (!PTHR_DCHECK(status, p >= 0 && p < V && (int)parent[p] < V)) { ok = false; return x; }
 #endif
         const int gp = parent[p];
-        if (gp != p) parent[x] = (uint16_t)gp;   // path halving: gp is an ancestor of x
+        if (gp != p) parent[x] = (Parent)gp;   // path halving: gp is an ancestor of x
         x = gp;
     }
     ok = false;
@@ -90,7 +93,8 @@ __device__ __forceinline__ int find_root(volatile uint16_t *parent, int x, int c
 // is done: the forest no longer changes, but other threads are writing the
 // final roots, and a path-halving store could replace a final root with an
 // intermediate ancestor after its owner wrote it.
-__device__ __forceinline__ int find_root_readonly(volatile uint16_t *parent, int x, int cap, bool &ok,
+template <typename Parent>
+__device__ __forceinline__ int find_root_readonly(volatile Parent *parent, int x, int cap, bool &ok,
                                                   uint32_t *status, int V) {
     for (int it = 0; it < cap; ++it) {
         const int p = parent[x];
@@ -104,16 +108,22 @@ __device__ __forceinline__ int find_root_readonly(volatile uint16_t *parent, int
     return x;
 }
 
-__device__ __forceinline__ void unite(volatile uint16_t *parent, int a, int b, int cap, bool &ok,
+__device__ __forceinline__ uint16_t swap_root(volatile uint16_t *p, uint16_t a, uint16_t b) {
+    return atomicCAS(const_cast<unsigned short *>((volatile unsigned short *)p), a, b);
+}
+__device__ __forceinline__ int swap_root(volatile int *p, int a, int b) {
+    return atomicCAS(const_cast<int *>(p), a, b);
+}
+
+template <typename Parent>
+__device__ __forceinline__ void unite(volatile Parent *parent, int a, int b, int cap, bool &ok,
                                       uint32_t *status, int V) {
     for (int it = 0; it < cap; ++it) {
         a = find_root(parent, a, cap, ok, status, V);
         b = find_root(parent, b, cap, ok, status, V);
         if (!ok || a == b) return;
         if (a < b) { const int t = a; a = b; b = t; }   // hook the larger root a under b
-        const unsigned short old = atomicCAS(const_cast<unsigned short *>((volatile unsigned short *)&parent[a]),
-                                             (unsigned short)a, (unsigned short)b);
-        if (old == (unsigned short)a) return;
+        if (swap_root(&parent[a], (Parent)a, (Parent)b) == (Parent)a) return;
     }
     ok = false;
 }
@@ -147,6 +157,53 @@ __device__ __forceinline__ int bond_int(float j, bool negated, uint32_t &bad) {
     const int v = __float_as_int(fmaf(j, 262144.f, 12582912.f)) - 0x4B400000;
     bad |= (float)v * 3.814697265625e-06f != j;
     return negated ? -v : v;
+}
+
+// Adds the sums of J s_i s_j over the forward bonds of row r after the flips to
+// Ea (clone a) and Eb (clone b): FP32 pairs over half a row's bonds (at most 36
+// terms), added up in FP64.  (The low part of one pair over a lane's 3 L^2
+// bonds would itself round: L = 24 2e-14 of the energy, 2e-16 so.)  U: sites
+// whose couplings are loaded together.
+template <int L, int U, typename Row>
+__device__ __forceinline__ void row_energies(const float *J, const Row *qs, const Row *as, const Row *Fs, int r,
+                                             double &Ea, double &Eb) {
+    constexpr int V = L * L * L;
+    const int y = r % L, z = r / L;
+    const int ry = (y + 1 == L ? 0 : y + 1) + L * z, rz = y + L * (z + 1 == L ? 0 : z + 1);
+    const uint32_t ar = as[r] ^ Fs[r], ay = as[ry] ^ Fs[ry], az = as[rz] ^ Fs[rz];
+    const uint32_t br = ar ^ qs[r], by = ay ^ qs[ry], bz = az ^ qs[rz];
+    const uint32_t na[3] = {ar ^ rot_next<L>(ar), ar ^ ay, ar ^ az};
+    const uint32_t nb[3] = {br ^ rot_next<L>(br), br ^ by, br ^ bz};
+#pragma unroll 1
+    for (int x0 = 0; x0 < L; x0 += L / 2) {
+        float h = 0.f, l = 0.f, h2 = 0.f, l2 = 0.f;
+#pragma unroll U
+        for (int x = x0; x < x0 + L / 2; ++x) {
+#pragma unroll
+            for (int d = 0; d < 3; ++d) {
+                const float j = __ldg(J + d * V + L * r + x);
+                two_sum_acc(h, l, ((na[d] >> x) & 1u) ? -j : j);
+                two_sum_acc(h2, l2, ((nb[d] >> x) & 1u) ? -j : j);
+            }
+        }
+        Ea += (double)h + (double)l;
+        Eb += (double)h2 + (double)l2;
+    }
+}
+
+// flip bits of bit word i of a lattice in the bit layout, from its flip rows
+template <int L, typename Row>
+__device__ __forceinline__ uint32_t flip_bits(const Row *Fs, int i) {
+    constexpr int ROWS = Geom<L>::ROWS, W = Geom<L>::W;
+    uint32_t m = 0;
+#pragma unroll
+    for (int t = 0; t < 8; ++t) {
+        const int w = 8 * i + t;
+        const int c = w / (ROWS * W), g = w - c * ROWS * W;
+        const int r = g / W, j = g - r * W;
+        m |= (compact_bits((uint32_t)Fs[r] >> ((c + r % L + r / L) & 1)) >> (4 * j) & 0xFu) << (4 * t);
+    }
+    return m;
 }
 
 // ------------------------------------------------------------ items
@@ -194,9 +251,9 @@ __device__ __forceinline__ bool cluster_sign(const PairItem &p, int label) {
 //     root is the smallest site index of its cluster (the canonical label).
 //     An edge whose left neighbours in both rows are in the same two runs is
 //     implied by that neighbouring edge and skipped; x = 0 never skips.
-template <int L, typename Row>
-__device__ __noinline__ bool union_find_pair(const ClusterArgs &a, const PairItem &p, int target, const Row *qs,
-                                             Row *Fs, uint16_t *parent, uint16_t *cnt, int cap, PairStats &st) {
+template <int L, typename Row, typename Parent>
+__device__ __forceinline__ bool union_find(const ClusterArgs &a, const PairItem &p, int target, const Row *qs,
+                                           Row *Fs, Parent *parent, uint16_t *cnt, int cap, PairStats &st) {
     constexpr int V = L * L * L;
     constexpr uint32_t M = (1u << L) - 1u;
     __shared__ int s_ok, s_nclus, s_top[2][32];
@@ -213,12 +270,12 @@ __device__ __noinline__ bool union_find_pair(const ClusterArgs &a, const PairIte
         int root = i0;
         for (int x = 0; x < L; ++x) {
             if ((st_ >> x) & 1u) root = i0 + x;
-            parent[i0 + x] = (uint16_t)((wrap && x >= last) ? i0 : root);
+            parent[i0 + x] = (Parent)((wrap && x >= last) ? i0 : root);
         }
     }
     __syncthreads();
     bool ok = true;
-    volatile uint16_t *vp = parent;
+    volatile Parent *vp = parent;
     for (int tsk = tid; tsk < 2 * L * L; tsk += T) {
         const int r = tsk >> 1;
         const int y = r % L, z = r / L;
@@ -234,7 +291,7 @@ __device__ __noinline__ bool union_find_pair(const ClusterArgs &a, const PairIte
     __syncthreads();
     // every site points straight at its root; only final roots are written
     // here (no path halving), so after the barrier parent[i] is the root
-    for (int i = tid; i < V; i += T) parent[i] = (uint16_t)find_root_readonly(vp, i, cap, ok, b.status, V);
+    for (int i = tid; i < V; i += T) parent[i] = (Parent)find_root_readonly(vp, i, cap, ok, b.status, V);
     if (!ok) s_ok = 0;
     __syncthreads();
     if (!s_ok) return false;
@@ -285,6 +342,13 @@ __device__ __noinline__ bool union_find_pair(const ClusterArgs &a, const PairIte
     }
     __syncthreads();
     return true;
+}
+
+// The same as a call of its own, so that its registers are not the floods'.
+template <int L, typename Row>
+__device__ __noinline__ bool union_find_pair(const ClusterArgs &a, const PairItem &p, int target, const Row *qs,
+                                             Row *Fs, uint16_t *parent, uint16_t *cnt, int cap, PairStats &st) {
+    return union_find<L, Row, uint16_t>(a, p, target, qs, Fs, parent, cnt, cap, st);
 }
 
 // A lane's rows hold the unlabelled sites of both signs of q: for L <= 16 the
@@ -435,29 +499,7 @@ __device__ __forceinline__ void finish_pair(const ClusterArgs &a, const PairItem
     const bool exact_E = ((off >> (sub * LN)) & (unsigned)((1ull << LN) - 1ull)) == 0u;
     double Ea = 0.0, Eb = 0.0;
     if (go && !exact_E && yl < L) {
-        for (int z = 0; z < L; ++z) {
-            const int r = y + L * z, ry = yp + L * z, rz = y + L * ((z + 1) % L);
-            const uint32_t ar = as[r] ^ Fs[r], ay = as[ry] ^ Fs[ry], az = as[rz] ^ Fs[rz];
-            const uint32_t br = ar ^ qs[r], by = ay ^ qs[ry], bz = az ^ qs[rz];
-            const uint32_t na[3] = {ar ^ rot_next<L>(ar), ar ^ ay, ar ^ az};
-            const uint32_t nb[3] = {br ^ rot_next<L>(br), br ^ by, br ^ bz};
-            // FP32 pairs over half a row's bonds (at most 36 terms), added up
-            // in FP64: the low part of a sum over all of the lane's 3 L^2
-            // bonds would itself round (L = 24: 2e-14 of the energy, 2e-16 so)
-            for (int x0 = 0; x0 < L; x0 += L / 2) {
-                float h = 0.f, l = 0.f, h2 = 0.f, l2 = 0.f;
-                for (int x = x0; x < x0 + L / 2; ++x) {
-#pragma unroll
-                    for (int d = 0; d < 3; ++d) {
-                        const float j = __ldg(J + d * V + L * r + x);
-                        two_sum_acc(h, l, ((na[d] >> x) & 1u) ? -j : j);
-                        two_sum_acc(h2, l2, ((nb[d] >> x) & 1u) ? -j : j);
-                    }
-                }
-                Ea += (double)h + (double)l;
-                Eb += (double)h2 + (double)l2;
-            }
-        }
+        for (int z = 0; z < L; ++z) row_energies<L, L / 2>(J, qs, as, Fs, y + L * z, Ea, Eb);
     }
     for (int o = LN / 2; o > 0; o >>= 1) {
         dE += __shfl_xor_sync(FULLW, dE, o);
@@ -473,14 +515,7 @@ __device__ __forceinline__ void finish_pair(const ClusterArgs &a, const PairItem
     // ---- flip both clones
     if (b.bits) {
         for (int i = yl; i < LW / 8; i += LN) {
-            uint32_t m = 0;
-#pragma unroll
-            for (int t = 0; t < 8; ++t) {
-                const int w = 8 * i + t;
-                const int c = w / (ROWS * W), g = w - c * ROWS * W;
-                const int r = g / W, j = g - r * W;
-                m |= (compact_bits((uint32_t)Fs[r] >> ((c + r % L + r / L) & 1)) >> (4 * j) & 0xFu) << (4 * t);
-            }
+            const uint32_t m = flip_bits<L>(Fs, i);
             if (m) { A[i] ^= m; B[i] ^= m; }
         }
     } else if (yl < L) {
@@ -886,6 +921,210 @@ __device__ __forceinline__ void cluster_block(const ClusterArgs &a, int bid, uns
     }
 }
 
+// ------------------------------------------------------------ one block per pair
+// Launches of few pairs: a warp's flood is one serial chain, which such a
+// launch lasts as long as, while most of the GPU idles.  Here a whole block
+// labels its pair by the union-find over sites and shares out rows, bonds and
+// words among its threads; the pair's rows, int parents and sizes are all its
+// shared memory.  One sample, 28 pairs, thermalised (warps): L = 8 17 us (21
+// us), L = 16 26 us (46 us), L = 20 37 us (90 us), L = 24 58 us (142 us).
+// Registers for three blocks of 512 threads per SM to L = 18 (above it the
+// memory takes two): 64 registers cost 40% at L = 14, 336 pairs, 32 registers 8%.
+template <int L>
+constexpr size_t pair_smem() {
+    typedef typename RowType<(L > 16)>::T Row;
+    return (size_t)L * L * L * 4 + (((size_t)L * L * L * 2 + 15) & ~(size_t)15) + 3 * L * L * sizeof(Row) + 16;
+}
+
+template <int L>
+__global__ void __launch_bounds__(512, L <= 18 ? 3 : 2) pair_kernel(ClusterArgs a) {
+    using Gm = Geom<L>;
+    constexpr int V = Gm::V, ROWS = Gm::ROWS, W = Gm::W, LW = Gm::LAT_WORDS;
+    constexpr int CAP = 4 * V + 64;
+    typedef typename RowType<(L > 16)>::T Row;
+    extern __shared__ __align__(16) unsigned char smem[];
+    int *parent = reinterpret_cast<int *>(smem);
+    uint16_t *cnt = reinterpret_cast<uint16_t *>(parent + V);
+    Row *qs = reinterpret_cast<Row *>(smem + (size_t)V * 4 + (((size_t)V * 2 + 15) & ~(size_t)15));
+    Row *as = qs + ROWS, *Fs = as + ROWS;
+    __shared__ int s_n, s_target, s_part[16][2];
+    __shared__ double s_E[16][2];
+    __shared__ long long s_dE[16];
+    const Batch &b = a.b;
+    const int tid = threadIdx.x, T = blockDim.x, lane = tid & 31, wid = tid >> 5, nw = T >> 5;
+    const PairItem p = pair_item(a, blockIdx.x);
+    if (!p.live) return;                                 // the same for the block
+    uint32_t *A = b.spins + ((size_t)p.s * b.NLAT + p.la) * b.lat_words;
+    uint32_t *B = b.spins + ((size_t)p.s * b.NLAT + p.lb) * b.lat_words;
+    if (tid == 0) { s_n = 0; s_target = -1; }
+    for (int r = tid; r < ROWS; r += T) {
+        const int p0 = (r % L + r / L) & 1;
+        uint32_t av, bv;
+        if (b.bits) {
+            av = row_of_bits<L>(A, r, p0);
+            bv = row_of_bits<L>(B, r, p0);
+        } else {
+            uint32_t wa[2][W], wb[2][W];
+#pragma unroll
+            for (int c = 0; c < 2; ++c) {
+                load_words<W>(A + (c * ROWS + r) * W, wa[c]);
+                load_words<W>(B + (c * ROWS + r) * W, wb[c]);
+            }
+            av = row_of_words<L>(wa, p0);
+            bv = row_of_words<L>(wb, p0);
+        }
+        as[r] = (Row)av;
+        qs[r] = (Row)(av ^ bv);
+    }
+    __syncthreads();
+    // ---- single-cluster move: the floor(u*n)-th q = -1 site in site order
+    if (b.cluster_mode != PTHR_CLUSTER_ACU && !a.label_only) {
+        const int chunk = (ROWS + T - 1) / T;
+        const int lo = min(ROWS, tid * chunk), hi = min(ROWS, lo + chunk);
+        int my = 0;
+        for (int r = lo; r < hi; ++r) my += __popc((uint32_t)qs[r]);
+        int incl = my;
+        for (int o = 1; o < 32; o <<= 1) {
+            const int t = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += t;
+        }
+        if (lane == 31) s_part[wid][0] = incl;
+        __syncthreads();
+        int before = incl - my, n = 0;
+        for (int w = 0; w < nw; ++w) {
+            if (w < wid) before += s_part[w][0];
+            n += s_part[w][0];
+        }
+        if (n > 0) {
+            const uint32_t w = philox_word0(p.seed, 0u, p.pair_id, p.emcs, TAG_SINGLE);
+            const int want = (int)(((unsigned long long)(w >> 8) * (unsigned long long)n) >> 24);
+            if (want >= before && want < before + my) {
+                for (int r = lo; r < hi; ++r) {
+                    uint32_t v = qs[r];
+                    const int c = __popc(v);
+                    if (want < before + c) {
+                        for (int m = want - before; m > 0; --m) v &= v - 1u;
+                        s_target = L * r + __ffs(v) - 1;
+                        break;
+                    }
+                    before += c;
+                }
+            }
+        }
+        __syncthreads();
+    }
+    PairStats st{0, 0, 0};
+    if (!union_find<L, Row, int>(a, p, s_target, qs, Fs, parent, cnt, CAP, st)) {
+        if (tid == 0) set_status(b.status, STATUS_NOCONVERGE);
+        return;
+    }
+    if (a.label_only) return;
+    // ---- energies from the cut bonds (see finish_pair)
+    const float *J = b.J + (size_t)p.s * 3 * V;
+    int sum = 0, nflip = 0;                              // at most 2 rows of 3 L terms below 2^23
+    uint32_t bad = 0;
+    for (int r = tid; r < ROWS; r += T) {
+        const int y = r % L, z = r / L;
+        const int ry = (y + 1 == L ? 0 : y + 1) + L * z, rz = y + L * (z + 1 == L ? 0 : z + 1);
+        const uint32_t f = Fs[r], av = as[r];
+        const uint32_t cut[3] = {f ^ rot_next<L>(f), f ^ Fs[ry], f ^ Fs[rz]};
+        const uint32_t neg[3] = {av ^ rot_next<L>(av), av ^ as[ry], av ^ as[rz]};
+        nflip += __popc(f);
+#pragma unroll
+        for (int d = 0; d < 3; ++d)
+            for (uint32_t cb = cut[d]; cb; cb &= cb - 1u) {
+                const int x = __ffs(cb) - 1;
+                sum += bond_int(__ldg(J + d * V + L * r + x), (neg[d] >> x) & 1u, bad);
+            }
+    }
+    const bool exact_E = __syncthreads_or(bad != 0u) == 0;
+    double ea = 0.0, eb = 0.0;
+    if (!exact_E)
+#pragma unroll 1
+        for (int r = tid; r < ROWS; r += T) row_energies<L, 1>(J, qs, as, Fs, r, ea, eb);
+    // (a warp's sums of both, below 2^31 where cut into 16-bit halves)
+    int hi = __reduce_add_sync(0xffffffffu, sum >> 12);
+    const unsigned lo = __reduce_add_sync(0xffffffffu, (unsigned)(sum & 0xFFF));
+    nflip = __reduce_add_sync(0xffffffffu, nflip);
+    if (!exact_E)
+        for (int o = 16; o > 0; o >>= 1) {
+            ea += __shfl_xor_sync(0xffffffffu, ea, o);
+            eb += __shfl_xor_sync(0xffffffffu, eb, o);
+        }
+    if (lane == 0) {
+        s_dE[wid] = (long long)hi * 4096 + (long long)lo;
+        s_part[wid][0] = nflip;
+        s_E[wid][0] = ea;
+        s_E[wid][1] = eb;
+    }
+    // ---- flip both clones
+    if (b.bits) {
+        for (int i = tid; i < LW / 8; i += T) {
+            const uint32_t m = flip_bits<L>(Fs, i);
+            if (m) { A[i] ^= m; B[i] ^= m; }
+        }
+    } else {
+        for (int r = tid; r < ROWS; r += T) {
+            const uint32_t f = Fs[r];
+            if (!f) continue;
+#pragma unroll
+            for (int c = 0; c < 2; ++c) {
+                uint32_t wa[W], wb[W];
+                load_words<W>(A + (c * ROWS + r) * W, wa);
+                load_words<W>(B + (c * ROWS + r) * W, wb);
+                const uint32_t v = f >> ((c + r % L + r / L) & 1);
+#pragma unroll
+                for (int j = 0; j < W; ++j) {
+                    wa[j] ^= word_flips(v, j);
+                    wb[j] ^= word_flips(v, j);
+                }
+                store_words<W>(A + (c * ROWS + r) * W, wa);
+                store_words<W>(B + (c * ROWS + r) * W, wb);
+            }
+        }
+    }
+    __syncthreads();
+    if (tid == 0) {
+        long long dE = 0;
+        int flips = 0;
+        double Ea = 0.0, Eb = 0.0;
+        for (int w = 0; w < nw; ++w) {
+            dE += s_dE[w];
+            flips += s_part[w][0];
+            Ea += s_E[w][0];
+            Eb += s_E[w][1];
+        }
+        double *E = b.E + (size_t)p.s * b.NLAT;
+        if (exact_E) {
+            const double dH = (double)(2 * dE) * (1.0 / 262144.0);
+            E[p.la] += dH;
+            E[p.lb] -= dH;
+        } else {
+            E[p.la] = -Ea;
+            E[p.lb] = -Eb;
+        }
+        long long *cs = b.cstat + (((size_t)p.s * b.NPAIR + p.P) * b.NT + p.k) * 4;
+        cs[0] = st.nclus;
+        cs[1] = st.top1;
+        cs[2] = st.top2;
+        cs[3] = flips;
+    }
+}
+
+template <int L>
+cudaError_t launch_pairs_L(const ClusterArgs &a, int threads, cudaStream_t st) {
+    static bool configured = false;
+    if (!configured) {
+        cudaError_t e = allow_max_dynamic_smem(pair_kernel<L>);
+        if (e != cudaSuccess) return e;
+        configured = true;
+    }
+    const int blocks = a.sample_count * a.b.NPAIR * a.b.n_acu;
+    if (blocks <= 0) return cudaSuccess;
+    pair_kernel<L><<<blocks, threads, pair_smem<L>(), st>>>(a);
+    return cudaGetLastError();
+}
+
 template <int L>
 __global__ void __launch_bounds__(CLUSTER_MAX_THREADS, L <= 8 || L > 16 ? 4 : 5) cluster_kernel(ClusterArgs a) {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -947,6 +1186,13 @@ cudaError_t launch_group_cluster(const GroupClusterArgs &g, int blocks, int thre
     }
     group_cluster_kernel<<<blocks, threads, smem, st>>>(g);
     return cudaGetLastError();
+}
+
+cudaError_t launch_cluster_pairs(const ClusterArgs &a, int threads, cudaStream_t st) {
+#define X(LL) if (a.b.L == LL) return launch_pairs_L<LL>(a, threads, st);
+    PTHR_FOR_EACH_L(X)
+#undef X
+    return cudaErrorInvalidValue;
 }
 
 size_t cluster_smem_bytes_for(int L, int threads) {

@@ -41,6 +41,8 @@ struct ClusterArgs {
 };
 constexpr int CLUSTER_MAX_THREADS = 128;   // per block: its warps work on pairs of their own
 cudaError_t launch_cluster(const ClusterArgs &a, int threads, cudaStream_t st);
+// one block per pair (iter_cap is not used: the bound 4V + 64)
+cudaError_t launch_cluster_pairs(const ClusterArgs &a, int threads, cudaStream_t st);
 size_t cluster_smem_bytes_for(int L, int threads);
 int cluster_blocks_for(int L, int pairs, int threads);   // blocks for that many pairs
 
