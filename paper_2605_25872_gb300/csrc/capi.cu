@@ -913,9 +913,22 @@ pthr_status group_fused_emcs(pthr_batch *const *batches, int n, cudaStream_t st,
     GroupSweepArgs gs{};
     GroupClusterArgs gc{};
     GroupBatchArgs gw{}, gm{};
-    int cl_threads = 32;   // one block size: the largest of the group
-    for (int i = 0; i < n; ++i)
-        if (cluster_threads_of(batches[i]) > cl_threads) cl_threads = cluster_threads_of(batches[i]);
+    // cluster step: one form and one block size, the largest of the group.  A
+    // block per pair if each batch would run so and together they are few: the
+    // batches' shares of their own lines add up to less than one (five sizes, one
+    // sweep per EMCS: 1 sample of each 75 us, 97 with warps; 4 samples 88 and 100).
+    int cl_threads = 32, cl_pair_threads = 32;
+    double few = 0.0;
+    for (int i = 0; i < n; ++i) {
+        const pthr_batch *b = batches[i];
+        if (b->cfg.cluster_mode == PTHR_CLUSTER_OFF || b->dev.n_acu == 0) continue;
+        const int pairs = b->cfg.n_samples * b->dev.NPAIR * b->dev.n_acu, t = pair_block_threads(b, pairs);
+        few += t > 0 ? (double)pairs / cluster_pair_limit(b->cfg.L) : 1.0;
+        if (t > cl_pair_threads) cl_pair_threads = t;
+        if (cluster_threads_of(b) > cl_threads) cl_threads = cluster_threads_of(b);
+    }
+    const bool cl_pairs = few < 1.0;
+    if (cl_pairs) cl_threads = cl_pair_threads;
     int sw_threads = 32, sw_blocks = 0, cl_blocks = 0, w_blocks = 0, m_blocks = 0, w_threads = 32;
     size_t sw_smem = 0, cl_smem = 0, w_smem = 0, m_smem = 0;
     for (int ii = 0; ii < n; ++ii) {
@@ -940,8 +953,10 @@ pthr_status group_fused_emcs(pthr_batch *const *batches, int n, cudaStream_t st,
             gc.a[gc.n] = a;
             gc.off[gc.n] = cl_blocks;
             ++gc.n;
-            cl_blocks += cluster_blocks_for(c->L, c->n_samples * b->dev.NPAIR * b->dev.n_acu, cl_threads);
-            if (cluster_smem_bytes_for(c->L, cl_threads) > cl_smem) cl_smem = cluster_smem_bytes_for(c->L, cl_threads);
+            const int pairs = c->n_samples * b->dev.NPAIR * b->dev.n_acu;
+            cl_blocks += cl_pairs ? pairs : cluster_blocks_for(c->L, pairs, cl_threads);
+            const size_t smem = cl_pairs ? cluster_pair_smem_bytes_for(c->L) : cluster_smem_bytes_for(c->L, cl_threads);
+            if (smem > cl_smem) cl_smem = smem;
         }
         gw.b[gw.n] = b->dev;
         gw.flags[gw.n] = PTHR_SWAP_PT | (c->er_on ? PTHR_SWAP_ER : 0);
@@ -963,7 +978,7 @@ pthr_status group_fused_emcs(pthr_batch *const *batches, int n, cudaStream_t st,
     gm.off[gm.n] = m_blocks;
     if (sw_smem > 200 * 1024 || cl_smem > 200 * 1024) return PTHR_E_STATE;
     if (launch_group_sweep(gs, rule, sw_blocks, sw_threads, sw_smem, st) != cudaSuccess) return PTHR_E_CUDA;
-    if (launch_group_cluster(gc, cl_blocks, cl_threads, cl_smem, st) != cudaSuccess) return PTHR_E_CUDA;
+    if (launch_group_cluster(gc, cl_pairs, cl_blocks, cl_threads, cl_smem, st) != cudaSuccess) return PTHR_E_CUDA;
     if (launch_group_swap(gw, w_blocks, w_threads, w_smem, st) != cudaSuccess) return PTHR_E_CUDA;
     if (launch_group_measure(gm, m_blocks, m_smem, st) != cudaSuccess) return PTHR_E_CUDA;
     *launches = (sw_blocks > 0) + (cl_blocks > 0) + (w_blocks > 0) + (m_blocks > 0);

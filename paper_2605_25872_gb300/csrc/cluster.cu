@@ -937,12 +937,11 @@ constexpr size_t pair_smem() {
 }
 
 template <int L>
-__global__ void __launch_bounds__(512, L <= 18 ? 3 : 2) pair_kernel(ClusterArgs a) {
+__device__ __forceinline__ void pair_block(const ClusterArgs &a, int bid, unsigned char *smem) {
     using Gm = Geom<L>;
     constexpr int V = Gm::V, ROWS = Gm::ROWS, W = Gm::W, LW = Gm::LAT_WORDS;
     constexpr int CAP = 4 * V + 64;
     typedef typename RowType<(L > 16)>::T Row;
-    extern __shared__ __align__(16) unsigned char smem[];
     int *parent = reinterpret_cast<int *>(smem);
     uint16_t *cnt = reinterpret_cast<uint16_t *>(parent + V);
     Row *qs = reinterpret_cast<Row *>(smem + (size_t)V * 4 + (((size_t)V * 2 + 15) & ~(size_t)15));
@@ -952,7 +951,7 @@ __global__ void __launch_bounds__(512, L <= 18 ? 3 : 2) pair_kernel(ClusterArgs 
     __shared__ long long s_dE[16];
     const Batch &b = a.b;
     const int tid = threadIdx.x, T = blockDim.x, lane = tid & 31, wid = tid >> 5, nw = T >> 5;
-    const PairItem p = pair_item(a, blockIdx.x);
+    const PairItem p = pair_item(a, bid);
     if (!p.live) return;                                 // the same for the block
     uint32_t *A = b.spins + ((size_t)p.s * b.NLAT + p.la) * b.lat_words;
     uint32_t *B = b.spins + ((size_t)p.s * b.NLAT + p.lb) * b.lat_words;
@@ -1112,6 +1111,12 @@ __global__ void __launch_bounds__(512, L <= 18 ? 3 : 2) pair_kernel(ClusterArgs 
 }
 
 template <int L>
+__global__ void __launch_bounds__(512, L <= 18 ? 3 : 2) pair_kernel(ClusterArgs a) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    pair_block<L>(a, blockIdx.x, smem);
+}
+
+template <int L>
 cudaError_t launch_pairs_L(const ClusterArgs &a, int threads, cudaStream_t st) {
     static bool configured = false;
     if (!configured) {
@@ -1146,9 +1151,11 @@ cudaError_t launch_cluster_L(const ClusterArgs &a, int threads, cudaStream_t st)
 }
 
 // The cluster step of a mixed-L group (see kernels.cuh): the blocks of every
-// batch's cluster launch, dispatching on its lattice size; one block size for
-// the group.
-__global__ void __launch_bounds__(CLUSTER_MAX_THREADS, 5) group_cluster_kernel(GroupClusterArgs g) {
+// batch's cluster launch, dispatching on its lattice size; one block size and
+// one form for the group.
+template <bool PAIRS>
+__global__ void __launch_bounds__(PAIRS ? 512 : CLUSTER_MAX_THREADS, PAIRS ? 2 : 5)
+group_cluster_kernel(GroupClusterArgs g) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ ClusterArgs ca;
     const int i = group_member(g.off, g.n, (int)blockIdx.x);
@@ -1162,7 +1169,7 @@ __global__ void __launch_bounds__(CLUSTER_MAX_THREADS, 5) group_cluster_kernel(G
     __syncthreads();
     const int bid = (int)blockIdx.x - g.off[i];
     switch (ca.b.L) {
-#define X(LL) case LL: cluster_block<LL>(ca, bid, smem); break;
+#define X(LL) case LL: PAIRS ? pair_block<LL>(ca, bid, smem) : cluster_block<LL>(ca, bid, smem); break;
         X(4) X(6) X(8) X(10) X(12) X(14) X(16)
 #undef X
     }
@@ -1176,16 +1183,31 @@ int cluster_blocks_for(int L, int pairs, int threads) {
     return (pairs + slots - 1) / slots;
 }
 
-cudaError_t launch_group_cluster(const GroupClusterArgs &g, int blocks, int threads, size_t smem, cudaStream_t st) {
-    if (blocks <= 0) return cudaSuccess;
+template <bool PAIRS>
+static cudaError_t launch_group_cluster_form(const GroupClusterArgs &g, int blocks, int threads, size_t smem,
+                                             cudaStream_t st) {
     static bool configured = false;
     if (!configured) {
-        cudaError_t e = allow_max_dynamic_smem(group_cluster_kernel);
+        cudaError_t e = allow_max_dynamic_smem(group_cluster_kernel<PAIRS>);
         if (e != cudaSuccess) return e;
         configured = true;
     }
-    group_cluster_kernel<<<blocks, threads, smem, st>>>(g);
+    group_cluster_kernel<PAIRS><<<blocks, threads, smem, st>>>(g);
     return cudaGetLastError();
+}
+
+cudaError_t launch_group_cluster(const GroupClusterArgs &g, int pairs, int blocks, int threads, size_t smem,
+                                 cudaStream_t st) {
+    if (blocks <= 0) return cudaSuccess;
+    return pairs ? launch_group_cluster_form<true>(g, blocks, threads, smem, st)
+                 : launch_group_cluster_form<false>(g, blocks, threads, smem, st);
+}
+
+size_t cluster_pair_smem_bytes_for(int L) {
+#define X(LL) if (L == LL) return pair_smem<LL>();
+    PTHR_FOR_EACH_L(X)
+#undef X
+    return 0;
 }
 
 cudaError_t launch_cluster_pairs(const ClusterArgs &a, int threads, cudaStream_t st) {

@@ -43,6 +43,7 @@ constexpr int CLUSTER_MAX_THREADS = 128;   // per block: its warps work on pairs
 cudaError_t launch_cluster(const ClusterArgs &a, int threads, cudaStream_t st);
 // one block per pair (iter_cap is not used: the bound 4V + 64)
 cudaError_t launch_cluster_pairs(const ClusterArgs &a, int threads, cudaStream_t st);
+size_t cluster_pair_smem_bytes_for(int L);
 size_t cluster_smem_bytes_for(int L, int threads);
 int cluster_blocks_for(int L, int pairs, int threads);   // blocks for that many pairs
 
@@ -69,7 +70,9 @@ bool group_supports_L(int L);
 int group_sweep_kt(int L);                 // lattices per thread of the group sweep
 cudaError_t launch_group_sweep(const GroupSweepArgs &g, int rule, int blocks, int threads, size_t smem,
                                cudaStream_t st);
-cudaError_t launch_group_cluster(const GroupClusterArgs &g, int blocks, int threads, size_t smem, cudaStream_t st);
+// pairs: one block per pair, else warps hold whole pairs
+cudaError_t launch_group_cluster(const GroupClusterArgs &g, int pairs, int blocks, int threads, size_t smem,
+                                 cudaStream_t st);
 cudaError_t launch_group_swap(const GroupBatchArgs &g, int blocks, int threads, size_t smem, cudaStream_t st);
 cudaError_t launch_group_measure(const GroupBatchArgs &g, int blocks, size_t smem, cudaStream_t st);
 size_t measure_smem_bytes_for(int L, int n_replicas);
