@@ -185,38 +185,53 @@ int default_k(const pthr_config *c, int total_entries) {
 // 3.71 ms, 60 sweeps of 16 clones 2.47 against 3.04 ms).
 constexpr int RES_HOIST_SWEEPS = 16;
 
+// Lattices per block where `total` lattices of each of `samples` samples fill
+// fewer blocks of K than SMs; lanes: lattice lanes of a block.  A block of few
+// lattices is staged for few updates, which a launch of few sweeps does not
+// earn back (one sweep, L = 8, 128 samples of 16 temperatures: 20 us with K = 64,
+// 33 with 4, and 11 and 25 per launch of three batches on three streams), so
+// K shrinks
+//  - while all blocks still have an SM each, those of one or a few sweeps with
+//    more than four lattices leaving a part of the SMs to other launches;
+//  - further, to blocks that take turns, where their form gains more than the
+//    staging costs (one launch alone / per launch of three, us):
+//    four lattices, whose threads keep the couplings in registers, in reservoir
+//    launches (RES_HOIST_SWEEPS); with the heat bath at one or two lanes (L = 10,
+//    75 samples, 3 sweeps 150 / 150 with K = 64, 123 / 112); from 10 sweeps on
+//    with Metropolis at one lane (L = 12, 18 samples 113 / 68 and 81 / 65) and
+//    with MicSA, whose draws serve four lattices, at two lanes or up to half the
+//    SMs (L = 16, 9 samples 120 / 57 and 70 / 61; 18 samples 120 / 110, 134 / 121);
+//    four lanes of four with the heat bath and MicSA at more lanes (L = 6, 150
+//    samples, 10 sweeps with MicSA 52 / 46 with K = 64, 53 / 36);
+//    32 lattices with Metropolis at more lanes, from 10 sweeps on (L = 10, 75
+//    samples 266 / 213 and 273 / 200; L = 8, 150 samples 75 / 69 and 73 / 66),
+//    8 at L <= 4 (150 samples 26 / 19 and 27 / 18; 32 lattices 28 / 22).
+int few_lattices(const pthr_config *c, int K, int total, int samples, int sweeps, int lanes) {
+    const auto blocks = [&](int k) { return samples * ((total + k - 1) / k); };
+    const int large = blocks(K);
+    if (large >= GPU_SMS || K <= 4 || sweeps <= 0) return K;
+    int most = K;
+    if (lanes > 2 && c->update_rule != PTHR_METROPOLIS) most = 16;
+    else if (sweeps >= RES_HOIST_SWEEPS || c->update_rule == PTHR_HEATBATH) most = 4;
+    else if (c->update_rule == PTHR_MICSA) most = sweeps >= 10 && (lanes == 2 || large <= GPU_SMS / 2) ? 4 : K;
+    else if (sweeps >= 10) most = lanes == 1 ? 4 : (lanes < 32 ? 32 : 8);
+    if (most > K) most = K;
+    const int sms = sweeps >= 10 ? GPU_SMS : GPU_SMS * 2 * sweeps / (2 * sweeps + 1);
+    for (int k = 4; k < most; k *= 2)
+        if (blocks(k) <= (k == 4 ? GPU_SMS : sms)) return k;
+    return most;
+}
+
 // forced_kt > 0: lattices per thread fixed (the mixed-L group sweep compiles
 // one value per lattice size); the lattices per block then follow from it.
-// samples, res_sweeps: the launch's samples and reservoir sweeps; with any,
-// its long blocks are the reservoir's (240 sweeps per EMCS against 10).
-SweepShape sweep_shape(const pthr_batch *b, int forced_kt, int samples, int res_sweeps) {
+// samples, pt_sweeps, res_sweeps: of the launch.
+SweepShape sweep_shape(const pthr_batch *b, int forced_kt, int samples, int pt_sweeps, int res_sweeps) {
     const pthr_config *c = &b->cfg;
-    const bool res = res_sweeps > 0;
     SweepShape sh{};
     const int npt = c->n_replicas * c->n_temps;
     const int nres = c->n_replicas * (c->n_res > 0 ? c->n_res : 1);
     sh.K_pt = default_k(c, npt);
     sh.K_res = default_k(c, nres);
-    const int long_blocks = samples * (res ? (nres + sh.K_res - 1) / sh.K_res : (npt + sh.K_pt - 1) / sh.K_pt);
-    const bool small = long_blocks < GPU_SMS && forced_kt == 0;
-    if (small) {
-        // fewer long blocks than SMs: smaller blocks, and where a thread owns
-        // one group of a colour (L <= 16) few enough lattices per thread to
-        // keep its couplings in registers.  One EMCS alone / three batches on
-        // three streams: L = 14, 20 samples 0.81 / 0.62 ms (16 lattices per
-        // block: 3.05 / 1.02 ms); L = 18 MicSA, 24 samples 3.1 / 1.8 ms (5.5 /
-        // 1.9 ms; 4 lattices: 2.2 / 2.0 ms); L = 16, 64 samples' reservoir
-        // sweeps 1.62 ms (3.1 ms).  From one block per SM on the PT clones'
-        // larger blocks stay: their couplings are staged for more updates.
-        const bool one_group = sweep_groups_for(c->L) <= 512;
-        const int most = one_group ? 4 : 8;
-        if (sh.K_res > most) sh.K_res = most;
-        if (one_group && sh.K_pt > most) sh.K_pt = most;
-    }
-    if (b->tuning.pt_lattices_per_block > 0) sh.K_pt = b->tuning.pt_lattices_per_block;
-    if (b->tuning.res_lattices_per_block > 0) sh.K_res = b->tuning.res_lattices_per_block;
-    if (sh.K_pt > npt) sh.K_pt = npt;
-    if (sh.K_res > nres) sh.K_res = nres;
     const int G = sweep_groups_for(c->L);
     int Gt = G;
     if (G > 512) {
@@ -224,6 +239,41 @@ SweepShape sweep_shape(const pthr_batch *b, int forced_kt, int samples, int res_
             if (G % d == 0 && G / d <= 512) { Gt = G / d; break; }
     }
     sh.Gt = Gt;
+    // the kind that decides how long the launch lasts: the reservoir if one of its
+    // blocks outlasts by half an SM's share of the PT clones (240 sweeps against 10)
+    const bool res_long = 2 * (long)sh.K_res * res_sweeps * GPU_SMS > 3 * (long)samples * npt * pt_sweeps;
+    bool small = false;
+    if (forced_kt == 0 && Gt == G) {
+        // One EMCS alone / three batches on three streams: L = 14, 20 samples
+        // 0.81 / 0.62 ms (16 lattices per block: 3.05 / 1.02 ms); L = 16, 64
+        // samples' reservoir sweeps 1.62 ms (3.1 ms).  From one block per SM on
+        // the large blocks stay.
+        const int lanes = 512 / Gt;
+        // (the rules whose PT clones gain from small blocks in any launch)
+        const bool gains = c->update_rule == PTHR_HEATBATH || (c->update_rule == PTHR_MICSA && lanes > 2);
+        const bool by_res = res_long || (gains && res_sweeps > 0);
+        const int K = by_res ? sh.K_res : sh.K_pt, total = by_res ? nres : npt;
+        const int k = few_lattices(c, K, total, samples, by_res ? res_sweeps : pt_sweeps, lanes);
+        small = k < K || (by_res && (gains || res_sweeps >= RES_HOIST_SWEEPS) && samples * ((nres + K - 1) / K) < GPU_SMS);
+        int most = k > 4 ? k : 4;
+        if (small && sh.K_res > most) sh.K_res = most;
+        // few reservoir sweeps, one lane: the PT clones' blocks by their own sweeps
+        if (by_res && !gains && lanes == 1 && res_sweeps < RES_HOIST_SWEEPS)
+            most = few_lattices(c, sh.K_pt, npt, samples, pt_sweeps, lanes);
+        if (small && sh.K_pt > most) sh.K_pt = most;
+    } else if (forced_kt == 0 && res_long && samples * ((nres + sh.K_res - 1) / sh.K_res) < GPU_SMS && sh.K_res > 8) {
+        // several groups per thread (L > 16), the couplings reloaded for each:
+        // L = 18 MicSA, 24 samples 3.1 / 1.8 ms (16 lattices 5.5 / 1.9 ms; 4
+        // lattices 2.2 / 2.0 ms)
+        sh.K_res = 8;
+    }
+    if (b->tuning.pt_lattices_per_block > 0) sh.K_pt = b->tuning.pt_lattices_per_block;
+    if (b->tuning.res_lattices_per_block > 0) sh.K_res = b->tuning.res_lattices_per_block;
+    if (sh.K_pt > npt) sh.K_pt = npt;
+    if (sh.K_res > nres) sh.K_res = nres;
+    // a kind that is not swept does not shape the block (its lanes would idle)
+    if (pt_sweeps <= 0 && res_sweeps > 0 && sh.K_pt > sh.K_res) sh.K_pt = sh.K_res;
+    if (res_sweeps <= 0 && pt_sweeps > 0 && sh.K_res > sh.K_pt) sh.K_res = sh.K_pt;
     int P0 = 512 / Gt;
     if (b->tuning.sweep_threads > 0) P0 = b->tuning.sweep_threads / Gt;
     if (P0 < 1) P0 = 1;
@@ -279,13 +329,19 @@ SweepShape sweep_shape(const pthr_batch *b, int forced_kt, int samples, int res_
     return sh;
 }
 
+// The shape of a whole EMCS's sweep launch.
+SweepShape emcs_shape(const pthr_batch *b) {
+    const pthr_config *c = &b->cfg;
+    return sweep_shape(b, 0, c->n_samples, c->sweeps_per_emcs, c->er_on && c->n_res > 0 ? c->res_sweeps_per_emcs : 0);
+}
+
 struct SweepLaunch { SweepArgs a; int blocks, threads, KT; size_t smem; };
 
 // Arguments and shape of one sweep launch (blocks == 0: nothing to do).
 pthr_status sweep_launch(pthr_batch *b, int n_pt, int n_res, int first, int count, int pretherm,
                          int forced_kt, SweepLaunch *out) {
     const pthr_config *c = &b->cfg;
-    SweepShape sh = sweep_shape(b, forced_kt, count, c->n_res > 0 ? n_res : 0);
+    SweepShape sh = sweep_shape(b, forced_kt, count, pretherm ? 0 : n_pt, c->n_res > 0 ? n_res : 0);
     SweepArgs a{};
     a.b = b->dev;
     a.n_pt_sweeps = n_pt;
@@ -577,7 +633,7 @@ PTHR_API pthr_status pthr_set_tuning(pthr_batch *b, const pthr_tuning *t) {
         return fail(b, PTHR_E_INVAL, "tuning out of range");
     pthr_tuning old = b->tuning;
     b->tuning = nt;
-    SweepShape sh = sweep_shape(b, 0, b->cfg.n_samples, b->cfg.er_on ? b->cfg.res_sweeps_per_emcs : 0);
+    SweepShape sh = emcs_shape(b);
     const size_t smem = sweep_smem_bytes_for(b->cfg.L, sh.K_pt > sh.K_res ? sh.K_pt : sh.K_res);
     if (smem > 220 * 1024) {
         b->tuning = old;
@@ -606,7 +662,7 @@ PTHR_API pthr_status pthr_set_update_rule(pthr_batch *b, int rule) {
 
 PTHR_API pthr_status pthr_get_tuning(const pthr_batch *b, pthr_tuning *t) {
     if (!b || !t) return fail(nullptr, PTHR_E_INVAL, "NULL argument");
-    SweepShape sh = sweep_shape(b, 0, b->cfg.n_samples, b->cfg.er_on ? b->cfg.res_sweeps_per_emcs : 0);
+    SweepShape sh = emcs_shape(b);
     t->pt_lattices_per_block = sh.K_pt;
     t->res_lattices_per_block = sh.K_res;
     t->sweep_threads = sh.threads;
