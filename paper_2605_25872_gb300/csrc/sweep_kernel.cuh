@@ -923,11 +923,17 @@ __device__ __forceinline__ bool res_block_in_registers(const SweepArgs &a, int b
     return a.KT_res == HOIST_KT && a.do_res && bid < a.sample_count * a.res_tasks;
 }
 
-template <int L, int RULE, int KT>
+// TWO_FORMS: the reservoir's blocks with the couplings in registers beside PT
+// blocks of KT.  A kernel of its own, for launches that have such blocks: the two
+// forms share a register budget (L = 16 heat bath: 80 bytes of spills, 12 alone)
+// and are more code to fetch (PT clones alone, in the kernel of both forms and in
+// its own: L = 12 MicSA, one sweep, 25 samples 32 and 23 us, 512 samples 843 and
+// 799 us; L = 16 Metropolis, 10 sweeps, 512 samples 3.71 and 3.57 ms).
+template <int L, int RULE, int KT, bool TWO_FORMS>
 __global__ void __launch_bounds__(SweepBounds<L, RULE>::threads, SweepBounds<L, RULE>::min_blocks)
 sweep_kernel(SweepArgs a) {
     extern __shared__ __align__(16) unsigned char smem[];
-    if constexpr (KT > HOIST_KT && res_in_registers<L, RULE>()) {
+    if constexpr (TWO_FORMS) {
         if (res_block_in_registers(a, blockIdx.x)) {
             sweep_block<L, RULE, HOIST_KT>(a, blockIdx.x, smem);
             return;
@@ -936,17 +942,26 @@ sweep_kernel(SweepArgs a) {
     sweep_block<L, RULE, KT>(a, blockIdx.x, smem);
 }
 
-template <int L, int RULE, int KT>
-cudaError_t launch_sweep_tpl(const SweepArgs &a, int blocks, int threads, size_t smem,
-                             cudaStream_t st) {
+template <int L, int RULE, int KT, bool TWO_FORMS>
+cudaError_t launch_sweep_form(const SweepArgs &a, int blocks, int threads, size_t smem, cudaStream_t st) {
     static bool configured = false;
     if (!configured) {
-        cudaError_t e = allow_max_dynamic_smem(sweep_kernel<L, RULE, KT>);
+        cudaError_t e = allow_max_dynamic_smem(sweep_kernel<L, RULE, KT, TWO_FORMS>);
         if (e != cudaSuccess) return e;
         configured = true;
     }
-    sweep_kernel<L, RULE, KT><<<blocks, threads, smem, st>>>(a);
+    sweep_kernel<L, RULE, KT, TWO_FORMS><<<blocks, threads, smem, st>>>(a);
     return cudaGetLastError();
+}
+
+template <int L, int RULE, int KT>
+cudaError_t launch_sweep_tpl(const SweepArgs &a, int blocks, int threads, size_t smem,
+                             cudaStream_t st) {
+    if constexpr (KT > HOIST_KT && res_in_registers<L, RULE>()) {
+        if (a.do_res && a.KT_res == HOIST_KT)
+            return launch_sweep_form<L, RULE, KT, true>(a, blocks, threads, smem, st);
+    }
+    return launch_sweep_form<L, RULE, KT, false>(a, blocks, threads, smem, st);
 }
 
 }  // namespace sweep_detail
