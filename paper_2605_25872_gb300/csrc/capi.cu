@@ -196,16 +196,15 @@ constexpr int RES_HOIST_SWEEPS = 16;
 //  - further, to blocks that take turns, where their form gains more than the
 //    staging costs (one launch alone / per launch of three, us):
 //    four lattices, whose threads keep the couplings in registers, in reservoir
-//    launches (RES_HOIST_SWEEPS); with the heat bath at one or two lanes (L = 10,
-//    75 samples, 3 sweeps 150 / 150 with K = 64, 123 / 112); from 10 sweeps on
+//    launches (RES_HOIST_SWEEPS); with the heat bath at one lane (L = 16, 13
+//    samples, 3 sweeps 90 / 59 with K = 16, 65 / 55); from 10 sweeps on
 //    with Metropolis at one lane (L = 12, 18 samples 113 / 68 and 81 / 65) and
 //    with MicSA, whose draws serve four lattices, at two lanes or up to half the
 //    SMs (L = 16, 9 samples 120 / 57 and 70 / 61; 18 samples 120 / 110, 134 / 121);
 //    four lanes of four with the heat bath and MicSA at more lanes (L = 6, 150
 //    samples, 10 sweeps with MicSA 52 / 46 with K = 64, 53 / 36);
-//    32 lattices with Metropolis at more lanes, from 10 sweeps on (L = 10, 75
-//    samples 266 / 213 and 273 / 200; L = 8, 150 samples 75 / 69 and 73 / 66),
-//    8 at L <= 4 (150 samples 26 / 19 and 27 / 18; 32 lattices 28 / 22).
+//    32 lattices with Metropolis at more lanes, from 10 sweeps on (L = 8, 150
+//    samples 75 / 69 with K = 64, 73 / 66), 8 at L <= 4 (150 samples 26 / 19 and 27 / 18; 32 lattices 28 / 22).
 int few_lattices(const pthr_config *c, int K, int total, int samples, int sweeps, int lanes) {
     const auto blocks = [&](int k) { return samples * ((total + k - 1) / k); };
     const int large = blocks(K);
@@ -239,6 +238,16 @@ SweepShape sweep_shape(const pthr_batch *b, int forced_kt, int samples, int pt_s
             if (G % d == 0 && G / d <= 512) { Gt = G / d; break; }
     }
     sh.Gt = Gt;
+    if (forced_kt == 0 && 512 / Gt == 2) {
+        // two lanes (L = 10): the variant of 32 lattices per thread keeps a flip
+        // count and an energy of each and spills 212 to 260 bytes (1024 samples of
+        // 24 temperatures, 10 sweeps / one: Metropolis 3.03 / 0.62 ms, with 16
+        // lattices per thread 2.79 / 0.51; heat bath 5.96 / 0.89, with 4, whose
+        // couplings stay in registers, 4.18 / 0.85)
+        const int most = c->update_rule == PTHR_HEATBATH ? 4 : 32;
+        if (sh.K_pt > most) sh.K_pt = most;
+        if (sh.K_res > most) sh.K_res = most;
+    }
     // the kind that decides how long the launch lasts: the reservoir if one of its
     // blocks outlasts by half an SM's share of the PT clones (240 sweeps against 10)
     const bool res_long = 2 * (long)sh.K_res * res_sweeps * GPU_SMS > 3 * (long)samples * npt * pt_sweeps;

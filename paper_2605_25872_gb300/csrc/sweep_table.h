@@ -19,8 +19,8 @@
     X(18, 1) X(18, 2) X(18, 4) X(18, 8) X(18, 16) \
     X(20, 1) X(20, 2) X(20, 4) X(20, 8) X(22, 1) X(22, 2) X(22, 4) X(24, 1) X(24, 2) X(24, 4)
 #define PTHR_SWEEP_HB_TABLE(X) \
-    X(2, 1) X(4, 2) X(6, 4) X(6, 8) X(8, 4) X(8, 8) X(10, 4) X(10, 32) X(12, 4) X(12, 32) X(14, 4) X(14, 32) \
-    X(16, 4) X(16, 32) X(18, 4) X(18, 16) X(20, 4) X(20, 8) X(22, 4) X(24, 4)
+    X(2, 1) X(4, 2) X(6, 4) X(6, 8) X(8, 4) X(8, 8) X(10, 4) X(10, 32) X(12, 4) X(12, 32) X(14, 4) X(14, 16) X(14, 32) \
+    X(16, 4) X(16, 16) X(16, 32) X(18, 4) X(18, 16) X(20, 4) X(20, 8) X(22, 4) X(24, 4)
 #define PTHR_SWEEP_MICSA_TABLE(X) \
     X(2, 1) X(4, 2) X(6, 4) X(6, 8) X(8, 4) X(8, 8) X(10, 4) X(10, 16) X(12, 4) X(12, 16) X(14, 4) X(14, 16) \
     X(16, 4) X(16, 16) X(18, 4) X(18, 16) X(20, 4) X(20, 8) X(22, 4) X(24, 4)

@@ -26,7 +26,7 @@ def pt_lattices(**kw):
     return Batch(BatchConfig(**kw)).get_tuning()["pt_lattices_per_block"]
 
 
-@pytest.mark.parametrize("L,S,NT,large", [(8, 128, 16, 64), (10, 64, 24, 64), (12, 25, 24, 16), (14, 12, 48, 16),
+@pytest.mark.parametrize("L,S,NT,large", [(8, 128, 16, 64), (10, 64, 24, 32), (12, 25, 24, 16), (14, 12, 48, 16),
                                           (16, 18, 32, 16)])
 def test_one_sweep_on_most_sms_keeps_the_large_blocks(L, S, NT, large):
     assert pt_lattices(L=L, n_samples=S, n_temps=NT) == large
@@ -61,3 +61,13 @@ def test_blocks_in_between_equal_one_lane(L, S, NT, n, rule):
         out.append((b.export_spins().cpu().numpy(), b.energies.cpu().numpy(), b.flips.cpu().numpy()))
     for x, y in zip(*out):
         np.testing.assert_array_equal(x, y)
+
+
+@pytest.mark.parametrize("L,rule,lattices", [(10, "metropolis", 16), (10, "heatbath", 4), (14, "heatbath", 16),
+                                             (16, "heatbath", 16)])
+def test_default_blocks_run_variants_of_fewer_lattices(L, rule, lattices):
+    # lattices per thread of a large launch of PT clones (test_sweep_registers_host.py:
+    # the variants of 32 at these sizes spill; L = 10 with the heat bath: couplings in registers)
+    t = Batch(BatchConfig(L=L, n_samples=160, n_temps=24, n_res=0, er_on=False, rule=rule)).get_tuning()
+    lanes = t["sweep_threads"] // (L * L * ((L // 2 + 3) // 4))
+    assert t["pt_lattices_per_block"] <= lattices * lanes

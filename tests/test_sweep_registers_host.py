@@ -1,5 +1,6 @@
 """The sweep kernel's variants, from the compiler's resource report: launches
-without reservoir blocks of their own form have a kernel of one form."""
+without reservoir blocks of their own form have a kernel of one form, and the
+variants that the default blocks run do not spill in it."""
 import os
 import re
 import shutil
@@ -30,3 +31,11 @@ def test_launches_of_one_form_have_a_kernel_of_their_own(tmp_path):
     assert len(spills(tmp_path, 12, "PTHR_MICSA", 16)) == 2
     assert len(spills(tmp_path, 16, "PTHR_HEATBATH", 32)) == 2
     assert len(spills(tmp_path, 12, "PTHR_METROPOLIS", 16)) == 1     # never two forms
+
+
+@pytest.mark.skipif(not os.path.exists(NVCC), reason="needs nvcc")
+@pytest.mark.parametrize("rule,variants", [("PTHR_METROPOLIS", [(10, 16), (14, 16), (16, 16)]),
+                                           ("PTHR_HEATBATH", [(14, 16), (16, 16)])])
+def test_default_variants_do_not_spill(tmp_path, rule, variants):
+    for L, kt in variants:
+        assert min(spills(tmp_path, L, rule, kt)) == 0, (L, kt)
