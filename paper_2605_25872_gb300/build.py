@@ -2,7 +2,8 @@
 
 Each translation unit is compiled by its own nvcc process (in parallel), then
 linked into paper_2605_25872_gb300/_build/libpthr.so with the CUDA runtime
-linked statically.
+linked statically.  The compiler's resource report (registers, spills and
+shared memory of every kernel) is kept beside it as ptxas.txt.
 """
 from __future__ import annotations
 
@@ -52,9 +53,7 @@ def build(force: bool = False, verbose: bool = False, extra_flags=(), debug: boo
     cc = nvcc()
     common = ["-O3", "-std=c++17", *ARCH, "-lineinfo", "-Xcompiler", "-fPIC",
               "-Xcompiler", "-fvisibility=hidden", "-I", os.path.join(ROOT, "include"),
-              "-I", CSRC, *extra_flags]
-    if verbose:
-        common += ["-Xptxas", "-v"]
+              "-I", CSRC, "-Xptxas", "-v", *extra_flags]
 
     def compile_one(src):
         obj = os.path.join(out_dir, src.replace(".cu", ".o"))
@@ -66,9 +65,11 @@ def build(force: bool = False, verbose: bool = False, extra_flags=(), debug: boo
 
     with ThreadPoolExecutor(max_workers=len(SOURCES)) as ex:
         results = list(ex.map(compile_one, SOURCES))
+    report = "".join(err for _, err in results)
     if verbose:
-        for _, err in results:
-            sys.stderr.write(err)
+        sys.stderr.write(report)
+    with open(os.path.join(out_dir, "ptxas.txt"), "w") as f:
+        f.write(report)
     tmp = lib + f".{os.getpid()}.tmp"
     cmd = [cc, "-shared", *ARCH, "-o", tmp, *[o for o, _ in results], "-cudart", "static"]
     r = subprocess.run(cmd, capture_output=True, text=True)

@@ -204,7 +204,8 @@ constexpr int RES_HOIST_SWEEPS = 16;
 //    four lanes of four with the heat bath and MicSA at more lanes (L = 6, 150
 //    samples, 10 sweeps with MicSA 52 / 46 with K = 64, 53 / 36);
 //    32 lattices with Metropolis at more lanes, from 10 sweeps on (L = 8, 150
-//    samples 75 / 69 with K = 64, 73 / 66), 8 at L <= 4 (150 samples 26 / 19 and 27 / 18; 32 lattices 28 / 22).
+//    samples 75 / 69 with K = 64, 73 / 66), 8 at L <= 4 (150 samples 26 / 19 and
+//    27 / 18; 32 lattices 28 / 22).
 int few_lattices(const pthr_config *c, int K, int total, int samples, int sweeps, int lanes) {
     const auto blocks = [&](int k) { return samples * ((total + k - 1) / k); };
     const int large = blocks(K);

@@ -1,41 +1,35 @@
-"""The sweep kernel's variants, from the compiler's resource report: launches
-without reservoir blocks of their own form have a kernel of one form, and the
-variants that the default blocks run do not spill in it."""
+"""The sweep kernel's variants in the compiler's resource report of the build:
+launches without reservoir blocks of their own form have a kernel of one form,
+and the variants that the default blocks run do not spill in it."""
 import os
 import re
-import shutil
-import subprocess
 
 import pytest
 
-from paper_2605_25872_gb300.build import ARCH, CSRC, ROOT
+from paper_2605_25872_gb300.build import BUILD, build
 
-NVCC = shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc"
-
-
-def spills(tmp_path, L, rule, kt):
-    """Bytes of spill stores of every kernel that launch_sweep_tpl<L, rule, kt> can launch."""
-    src = tmp_path / "v.cu"
-    src.write_text('#include "sweep_kernel.cuh"\nnamespace pthr {\ntemplate cudaError_t sweep_detail::launch_sweep_tpl'
-                   f"<{L}, {rule}, {kt}>(const SweepArgs &, int, int, size_t, cudaStream_t);\n}}\n")
-    r = subprocess.run([NVCC, "-O3", "-std=c++17", *ARCH, "-I", os.path.join(ROOT, "include"), "-I", CSRC, "-Xptxas", "-v",
-                        "-c", str(src), "-o", str(tmp_path / "v.o")], capture_output=True, text=True)
-    assert r.returncode == 0, r.stderr[-2000:]
-    found = re.findall(r"Function properties for (\S*sweep_kernel\S*)\s+\d+ bytes stack frame, (\d+) bytes spill", r.stderr)
-    assert found, r.stderr[-2000:]
-    return [int(n) for _, n in found]
+RULES = {"metropolis": 0, "heatbath": 1, "micsa": 2}
 
 
-@pytest.mark.skipif(not os.path.exists(NVCC), reason="needs nvcc")
-def test_launches_of_one_form_have_a_kernel_of_their_own(tmp_path):
-    assert len(spills(tmp_path, 12, "PTHR_MICSA", 16)) == 2
-    assert len(spills(tmp_path, 16, "PTHR_HEATBATH", 32)) == 2
-    assert len(spills(tmp_path, 12, "PTHR_METROPOLIS", 16)) == 1     # never two forms
+@pytest.fixture(scope="module")
+def spills():
+    """Bytes of spill stores by (L, rule, lattices per thread, both forms)."""
+    build()
+    with open(os.path.join(BUILD, "ptxas.txt")) as f:
+        report = f.read()
+    found = re.findall(r"Function properties for \S*sweep_kernelILi(\d+)ELi(\d+)ELi(\d+)ELb([01])E\S*\s+"
+                       r"\d+ bytes stack frame, (\d+) bytes spill", report)
+    return {(int(L), int(r), int(k), bool(int(two))): int(n) for L, r, k, two, n in found}
 
 
-@pytest.mark.skipif(not os.path.exists(NVCC), reason="needs nvcc")
-@pytest.mark.parametrize("rule,variants", [("PTHR_METROPOLIS", [(10, 16), (14, 16), (16, 16)]),
-                                           ("PTHR_HEATBATH", [(14, 16), (16, 16)])])
-def test_default_variants_do_not_spill(tmp_path, rule, variants):
+def test_launches_of_one_form_have_a_kernel_of_their_own(spills):
+    for L, rule, kt in ((12, "micsa", 16), (16, "heatbath", 32), (16, "metropolis", 16)):
+        assert (L, RULES[rule], kt, False) in spills and (L, RULES[rule], kt, True) in spills
+    assert (12, RULES["metropolis"], 16, True) not in spills     # never two forms
+
+
+@pytest.mark.parametrize("rule,variants", [("metropolis", [(10, 16), (14, 16), (16, 16)]),
+                                           ("heatbath", [(14, 16), (16, 16)])])
+def test_default_variants_do_not_spill(spills, rule, variants):
     for L, kt in variants:
-        assert min(spills(tmp_path, L, rule, kt)) == 0, (L, kt)
+        assert spills[L, RULES[rule], kt, False] == 0, (L, kt)
