@@ -305,6 +305,9 @@ SweepShape sweep_shape(const pthr_batch *b, int forced_kt, int samples, int pt_s
         // 0.96 ms against half of the lanes idle)
         int lanes = (sh.K_res + SWEEP_HOIST_KT - 1) / SWEEP_HOIST_KT;
         if (lanes * Gt < 128) lanes = (128 + Gt - 1) / Gt;
+        // (a caller's PT share keeps the lanes that it needs)
+        const int most = opts[nopt - 1];
+        if (b->tuning.pt_lattices_per_block > 0 && lanes * most < sh.K_pt) lanes = (sh.K_pt + most - 1) / most;
         if (P0 > lanes) P0 = lanes;
     }
     int Kmax = sh.K_pt > sh.K_res ? sh.K_pt : sh.K_res;

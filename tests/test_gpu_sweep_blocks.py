@@ -71,3 +71,10 @@ def test_default_blocks_run_variants_of_fewer_lattices(L, rule, lattices):
     t = Batch(BatchConfig(L=L, n_samples=160, n_temps=24, n_res=0, er_on=False, rule=rule)).get_tuning()
     lanes = t["sweep_threads"] // (L * L * ((L // 2 + 3) // 4))
     assert t["pt_lattices_per_block"] <= lattices * lanes
+
+
+@pytest.mark.parametrize("L,share", [(6, 64), (8, 64), (10, 48)])
+def test_a_callers_pt_share_is_kept_beside_reservoir_blocks(L, share):
+    cfg = BatchConfig(L=L, n_samples=160, n_temps=16, n_res=1)
+    b = Batch(cfg, tuning={"pt_lattices_per_block": share})
+    assert b.get_tuning()["pt_lattices_per_block"] == share
