@@ -50,9 +50,11 @@ def candidates(cfg: BatchConfig):
         if th:
             shape["sweep_threads"] = th
         yield shape
+    for ct in (32, 64, 128):                   # blocks whose warps hold whole pairs
+        yield {"cluster_threads": ct}
     V = cfg.L ** 3
-    for ct in (64, 128, 256, 384, 512):
-        if ct <= max(64, V // 2):
+    for ct in (192, 256, 384, 512):            # one block per pair
+        if ct <= V // 2:
             yield {"cluster_threads": ct}
 
 
