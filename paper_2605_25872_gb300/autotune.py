@@ -3,13 +3,15 @@
 It times whole EMCS (CUDA events on the batch's stream) for candidate shapes:
 lattices per sweep block for PT and reservoir clones, sweep threads, and
 cluster threads.  It does this on a scratch batch of the same configuration,
-keeps the fastest shape, and caches it per (configuration, GPU).  Shapes
+keeps the fastest shape, and caches it per (configuration, GPU, kernel sources).  Shapes
 never change results, because every random number is keyed by (sample,
 lattice, site, step), so tuning can run on synthetic couplings and the
 winner can be applied to any batch of that configuration.
 """
 from __future__ import annotations
 
+import functools
+import hashlib
 import itertools
 import json
 import os
@@ -18,14 +20,26 @@ import numpy as np
 
 from ._lib import PthrError
 from .batch import Batch, BatchConfig
+from .build import CSRC
 
 CACHE = os.path.join(os.path.dirname(os.path.abspath(__file__)), "_build", "tuning_cache.json")
+
+
+@functools.lru_cache(maxsize=None)
+def kernels_version(directory: str = CSRC) -> str:
+    """Hash of the library's sources: a shape is the fastest of the kernels it
+    was timed on."""
+    h = hashlib.sha1()
+    for f in sorted(os.listdir(directory)):
+        with open(os.path.join(directory, f), "rb") as fh:
+            h.update(f.encode() + b"\0" + fh.read())
+    return h.hexdigest()[:12]
 
 
 def _key(cfg: BatchConfig, device_name: str) -> str:
     d = dict(cfg.__dict__)
     d.pop("seed", None)
-    return device_name + "|" + json.dumps(d, sort_keys=True)
+    return device_name + "|" + kernels_version() + "|" + json.dumps(d, sort_keys=True)
 
 
 def sweep_lane_threads(L: int) -> list:
