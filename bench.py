@@ -498,11 +498,12 @@ def run_gpu(args):
 
 
 def kernel_version():
-    """Hash of the sweep kernel source: a stored DRAM-traffic figure is only
-    valid for the kernel it was measured on."""
+    """Hash of the sweep kernel source and of the rule that picks its launch
+    shape: a stored counter is only valid for the launch it was measured on."""
     import hashlib
     h = hashlib.sha1()
-    for f in ("sweep_kernel.cuh", "geometry.cuh", "sweep.cu", "sweep_table.h", "pthr_internal.cuh"):
+    for f in ("sweep_kernel.cuh", "geometry.cuh", "sweep.cu", "sweep_table.h", "pthr_internal.cuh",
+              "kernels.cuh", "capi.cu"):
         with open(os.path.join(ROOT, "paper_2605_25872_gb300", "csrc", f), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:12]
