@@ -225,11 +225,15 @@ __device__ __forceinline__ void set_status(uint32_t *status, uint32_t bit) {
 // sanitizer): a failed check latches STATUS_BOUNDS and evaluates to false,
 // and the caller then skips or clamps the access, so nothing outside a
 // buffer is read or written.  Release builds compile every check away.
+// PTHR_DCOVER latches in status word 1 that a checked path ran (COVER_*).
 #ifdef PTHR_DEBUG
 #define PTHR_DCHECK(status, cond) ((cond) ? true : (::pthr::set_status((status), ::pthr::STATUS_BOUNDS), false))
+#define PTHR_DCOVER(status, path) ::pthr::set_status((status) + 1, (path))
 #else
 #define PTHR_DCHECK(status, cond) true
+#define PTHR_DCOVER(status, path) ((void)0)
 #endif
+constexpr uint32_t COVER_SWEEP_SHARED = 1u, COVER_SWEEP_REGISTERS = 2u;   // couplings in shared memory, in registers
 
 // Supported linear sizes (template instantiations).
 #define PTHR_FOR_EACH_L(X) X(2) X(4) X(6) X(8) X(10) X(12) X(14) X(16) X(18) X(20) X(22) X(24)

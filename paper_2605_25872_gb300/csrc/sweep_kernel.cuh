@@ -407,6 +407,19 @@ struct SweepBounds {
         (RULE == PTHR_METROPOLIS && 65536 / (threads * 112) >= 2) ? 2 : 1;
 };
 
+// Range check of the debug build: group g of colour c, its words and couplings
+// in a lattice, and the thread's lattices in the block.
+template <int L, int KT>
+__device__ __forceinline__ bool sweep_in_range(const GroupGeo &q, int g, int c, int kbase, int K) {
+    using Gm = Geom<L>;
+    constexpr int W = Gm::W, ROWS = Gm::ROWS, LW = Gm::LAT_WORDS;
+    const int cm = ((c ^ 1) * ROWS + ROWS - 1) * W + W - 1;
+    return g >= 0 && g < Gm::G && q.own >= 0 && q.own < LW && q.xa >= 0 && q.xa < LW && q.wA >= 0 && q.wA < LW &&
+           q.wB >= 0 && q.wB < LW && q.yp >= 0 && q.yp < LW && q.ym >= 0 && q.ym < LW && q.zp >= 0 && q.zp < LW &&
+           q.zm >= 0 && q.zm < LW && 4 * q.own + 3 < Gm::LAT_BYTES && 4 * cm + 3 < Gm::LAT_BYTES &&
+           (kbase >= K || kbase + min(KT, K - kbase) <= MAXK);
+}
+
 // One block of the sweep launch: block `bid` of the launch described by a,
 // dynamic shared memory at smem.  Threads past the block's lattice lanes
 // (a launch shared with larger shapes) take part in the barriers only.
@@ -648,9 +661,24 @@ __device__ __forceinline__ void sweep_block(const SweepArgs &a, int bid, unsigne
     // launches with four lattices per block: L = 16, 64 samples 1.62 ms (2.05
     // ms); L = 4, one sample, KT = 1: 61 us (137 us).
     if (HOIST) {
+#ifdef PTHR_DEBUG
+        // a failed check leaves the thread (where lanes add up energies, its
+        // warp) with the barriers only, on group 0's words
+        if (tid == 0 && nsw > 0) PTHR_DCOVER(b.status, COVER_SWEEP_REGISTERS);
+        bool in = PTHR_DCHECK(b.status, (GP == 1 && sweep_in_range<L, KT>(qc0, g0, 0, kbase, K) &&
+                                         sweep_in_range<L, KT>(qc1, g0, 1, kbase, K)));
+        if (AT_ONCE) in = __all_sync(0xffffffffu, in) != 0;
+        if (!in) {
+            qc0 = group_geo<L>(0, 0);
+            qc1 = group_geo<L>(0, 1);
+        }
+        const int gJ = in ? g0 : 0;
+#else
+        const int gJ = g0;
+#endif
         f2 Jr[2][2][6];
-        sweep_couplings<L, RULE>(Js, qc0, g0, 0, Jr[0]);
-        sweep_couplings<L, RULE>(Js, qc1, g0, 1, Jr[1]);
+        sweep_couplings<L, RULE>(Js, qc0, gJ, 0, Jr[0]);
+        sweep_couplings<L, RULE>(Js, qc1, gJ, 1, Jr[1]);
         const uint32_t vmask = valid_mask<L>(g0 % W);
         uint32_t ahi, alo;
         mul_wide(0xD2511F53u, (uint32_t)g0, ahi, alo);
@@ -674,6 +702,12 @@ __device__ __forceinline__ void sweep_block(const SweepArgs &a, int bid, unsigne
             constexpr int c = decltype(colour)::value;
             constexpr bool ENERGY = decltype(energy)::value;
             const GroupGeo &q = c ? qc1 : qc0;
+#ifdef PTHR_DEBUG
+            if (!in) {
+                __syncthreads();
+                return;
+            }
+#endif
             // with one or two lattices the next words are drawn between
             // this half-sweep's loads and their use (two serial chains
             // side by side), else after it (the words of both would spill)
@@ -721,15 +755,10 @@ __device__ __forceinline__ void sweep_block(const SweepArgs &a, int bid, unsigne
             const int g = g0 + gi * Gt;
             const GroupGeo q = ONE_G ? (c ? qc1 : qc0) : group_geo<L>(g, c);
 #ifdef PTHR_DEBUG
-            {
-                const int cm = ((c ^ 1) * ROWS + ROWS - 1) * W + W - 1;
-                const bool in = g < G && q.own >= 0 && q.own < LW && q.xa >= 0 && q.xa < LW &&
-                                q.wA >= 0 && q.wA < LW && q.wB >= 0 && q.wB < LW && q.yp >= 0 &&
-                                q.yp < LW && q.ym >= 0 && q.ym < LW && q.zp >= 0 && q.zp < LW &&
-                                q.zm >= 0 && q.zm < LW && 4 * q.own + 3 < LB && 4 * cm + 3 < LB &&
-                                (kbase >= K || kbase + min(KT, K - kbase) <= MAXK);
-                if (!PTHR_DCHECK(b.status, in)) continue;
-            }
+            if (tid == 0) PTHR_DCOVER(b.status, COVER_SWEEP_SHARED);
+            bool in = PTHR_DCHECK(b.status, (sweep_in_range<L, KT>(q, g, c, kbase, K)));
+            if (AT_ONCE) in = __all_sync(0xffffffffu, in) != 0;   // the lanes that add up energies together
+            if (!in) continue;
 #endif
             uint32_t ahi, alo;
             mul_wide(0xD2511F53u, (uint32_t)g, ahi, alo);
