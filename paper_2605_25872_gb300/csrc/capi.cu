@@ -958,6 +958,11 @@ pthr_group *new_group(pthr_batch *const *batches, int n, cudaStream_t st, cudaGr
 
 namespace {
 
+// Dynamic shared memory of a group kernel: 227 KB less the static arrays of every
+// size's block (33.6 KB in the sweep: two forms for each of seven sizes).  A
+// group that needs more takes the per-batch graph.
+constexpr size_t GROUP_DYNAMIC_SMEM = 192 * 1024;
+
 // One EMCS of every batch as four launches in total (sweep, cluster move,
 // swap, measurement), each over the blocks of all batches; possible when
 // the batches share an update rule, their sizes are compiled into the group
@@ -1045,7 +1050,7 @@ pthr_status group_fused_emcs(pthr_batch *const *batches, int n, cudaStream_t st,
     gc.off[gc.n] = cl_blocks;
     gw.off[gw.n] = w_blocks;
     gm.off[gm.n] = m_blocks;
-    if (sw_smem > 200 * 1024 || cl_smem > 200 * 1024) return PTHR_E_STATE;
+    if (sw_smem > GROUP_DYNAMIC_SMEM || cl_smem > GROUP_DYNAMIC_SMEM) return PTHR_E_STATE;
     if (launch_group_sweep(gs, rule, sw_blocks, sw_threads, sw_smem, st) != cudaSuccess) return PTHR_E_CUDA;
     if (launch_group_cluster(gc, cl_pairs, cl_blocks, cl_threads, cl_smem, st) != cudaSuccess) return PTHR_E_CUDA;
     if (launch_group_swap(gw, w_blocks, w_threads, w_smem, st) != cudaSuccess) return PTHR_E_CUDA;

@@ -1,12 +1,13 @@
 """The sweep kernel's variants in the compiler's resource report of the build:
 launches without reservoir blocks of their own form have a kernel of one form,
-and the variants that the default blocks run do not spill in it."""
+and the variants that the default blocks run do not spill in it.  The group
+kernels' static and dynamic shared memory fit a block together."""
 import os
 import re
 
 import pytest
 
-from paper_2605_25872_gb300.build import BUILD, build
+from paper_2605_25872_gb300.build import BUILD, CSRC, build
 
 RULES = {"metropolis": 0, "heatbath": 1, "micsa": 2}
 
@@ -33,3 +34,15 @@ def test_launches_of_one_form_have_a_kernel_of_their_own(spills):
 def test_default_variants_do_not_spill(spills, rule, variants):
     for L, kt in variants:
         assert spills[L, RULES[rule], kt, False] == 0, (L, kt)
+
+
+def test_group_kernels_fit_their_dynamic_limit():
+    build()
+    with open(os.path.join(BUILD, "ptxas.txt")) as f:
+        report = f.read()
+    static = [int(n) for n in re.findall(
+        r"Compiling entry function '\S*group_(?:sweep|cluster)_kernel\S*' for \S+\n(?:.*\n)*?.*Used .* (\d+) bytes smem", report)]
+    assert len(static) == 5
+    with open(os.path.join(CSRC, "capi.cu")) as f:
+        limit = int(re.search(r"GROUP_DYNAMIC_SMEM = (\d+) \* 1024", f.read()).group(1)) * 1024
+    assert max(static) + limit <= 227 * 1024
