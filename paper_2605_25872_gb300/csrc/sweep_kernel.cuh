@@ -657,9 +657,13 @@ __device__ __forceinline__ void sweep_block(const SweepArgs &a, int bid, unsigne
     // takes about 900 + 775 KT cycles with them in shared memory), and a
     // half-sweep's random words are drawn before the barrier of the one before,
     // since they do not depend on spins.  More than four lattices per thread
-    // would spill (48 coupling registers of 128).  240-sweep reservoir
-    // launches with four lattices per block: L = 16, 64 samples 1.62 ms (2.05
-    // ms); L = 4, one sample, KT = 1: 61 us (137 us).
+    // would spill (48 coupling registers of 128; at L = 12 with the Metropolis
+    // rule two and four do, 76 and 168 bytes, since two blocks share an SM: one
+    // block of 163 registers takes 584 us alone and 449 us of three batches for an
+    // EMCS of 24 samples, two take 731 and 462, but 25 samples' 10 PT sweeps 114
+    // and 107 against 103 and 89).  240-sweep reservoir launches with four
+    // lattices per block: L = 16, 64 samples 1.62 ms (2.05 ms); L = 4, one
+    // sample, KT = 1: 61 us (137 us).
     if (HOIST) {
 #ifdef PTHR_DEBUG
         // a failed check leaves the thread (where lanes add up energies, its
@@ -789,9 +793,23 @@ __device__ __forceinline__ void sweep_block(const SweepArgs &a, int bid, unsigne
         }
         __syncthreads();
     };
+    // (the same half-sweeps as loops over sweeps and colours or as one loop: the
+    // compiler schedules Metropolis at one lane of whole warps, L = 12 and 16,
+    // better the first way and the others the second.  10 sweeps: L = 12, 1024
+    // samples 3.68 and 3.75 ms, L = 16, 512 samples 3.54 and 3.57, L = 14, 256
+    // samples 2.82 and 2.75, MicSA at L = 12, 512 samples 4.01 and 3.93; the group
+    // kernel's EMCS of five sizes 2.256 and 2.235)
     if (!HOIST && nsw > 0) {
-        for (int hs = 0; hs < 2 * nsw - 1; ++hs) half_sweep(hs >> 1, hs & 1, Const<0>());
-        half_sweep(nsw - 1, 1, Const<1>());
+        if (RULE == PTHR_METROPOLIS && MAY_HOIST && AT_ONCE && SweepBounds<L, RULE>::Gt >= 256) {
+            for (int sw = 0; sw < nsw; ++sw)
+                for (int c = 0; c < 2; ++c) {
+                    if (sw == nsw - 1 && c == 1) half_sweep(sw, c, Const<1>());
+                    else half_sweep(sw, c, Const<0>());
+                }
+        } else {
+            for (int hs = 0; hs < 2 * nsw - 1; ++hs) half_sweep(hs >> 1, hs & 1, Const<0>());
+            half_sweep(nsw - 1, 1, Const<1>());
+        }
     }
 
     // ---- energies (Eq. (1)) of the swept lattices and their flip counts
@@ -941,7 +959,8 @@ __device__ __forceinline__ void sweep_block(const SweepArgs &a, int bid, unsigne
 // on 512 groups (L = 16: one draw serves four lattices and the couplings come
 // by 16-byte loads; 10 PT and 240 reservoir sweeps of 512 samples 11.54 ms
 // with the one form, 11.89 ms with both; L = 14, 256 samples 6.65 and 6.61,
-// L = 10, 1024 samples 14.66 and 10.81).
+// L = 10, 1024 samples 14.66 and 10.81, L = 8 6.40 and 2.71: at fewer groups the
+// lanes of a large PT block would idle in the reservoir's).
 template <int L, int RULE>
 __host__ __device__ constexpr bool res_in_registers() {
     return Geom<L>::G <= 512 && SweepBounds<L, RULE>::min_blocks == 1 &&

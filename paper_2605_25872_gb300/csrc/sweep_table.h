@@ -4,7 +4,8 @@
 // 16, the largest that fits two blocks per SM without spilling).  Variants of
 // up to four keep the couplings in registers; launches of few blocks use them,
 // and the reservoir's blocks of larger launches run four inside the variants
-// of more.
+// of more.  32 per thread spill where a thread holds each lattice's flips and
+// energy to the end (L = 10, 14): a caller's shares reach them, no default.
 #pragma once
 
 #include <cuda_runtime.h>
