@@ -27,7 +27,8 @@
 // bound sets STATUS_NOCONVERGE and leaves the pair as it was.
 //
 // What bounds it: instruction issue and latency of the floods' serial chains
-// (40% issue active, DRAM below 10%); it reads and writes each clone once.
+// (40% issue active, DRAM 12% at L = 12); it reads each clone once and the rows
+// that flip twice.
 // Whole launch, thermalised, against the block-per-pair union-find over sites
 // that it replaces: L = 12, 28672 pairs 203 us (611 us); L = 16, 18432 pairs
 // 247 us (887 us); L = 8, 5120 pairs 36 us (44 us); at a random start, where
@@ -189,6 +190,16 @@ __device__ __forceinline__ void row_energies(const float *J, const Row *qs, cons
         Ea += (double)h + (double)l;
         Eb += (double)h2 + (double)l2;
     }
+}
+
+// The same over the rows z of one y; a call of its own, so that its registers are
+// not the flooding kernel's (L = 12, 256 samples, three batches, on the grid 50.4
+// us per launch inline, 48.3 so; 48.7 before the energies summed half rows).
+template <int L, typename Row>
+__device__ __noinline__ double2 column_energies(const float *J, const Row *qs, const Row *as, const Row *Fs, int y) {
+    double Ea = 0.0, Eb = 0.0;
+    for (int z = 0; z < L; ++z) row_energies<L, L / 2>(J, qs, as, Fs, y + L * z, Ea, Eb);
+    return make_double2(Ea, Eb);
 }
 
 // flip bits of bit word i of a lattice in the bit layout, from its flip rows
@@ -499,7 +510,9 @@ __device__ __forceinline__ void finish_pair(const ClusterArgs &a, const PairItem
     const bool exact_E = ((off >> (sub * LN)) & (unsigned)((1ull << LN) - 1ull)) == 0u;
     double Ea = 0.0, Eb = 0.0;
     if (go && !exact_E && yl < L) {
-        for (int z = 0; z < L; ++z) row_energies<L, L / 2>(J, qs, as, Fs, y + L * z, Ea, Eb);
+        const double2 e = column_energies<L>(J, qs, as, Fs, y);
+        Ea = e.x;
+        Eb = e.y;
     }
     for (int o = LN / 2; o > 0; o >>= 1) {
         dE += __shfl_xor_sync(FULLW, dE, o);
